@@ -118,6 +118,11 @@ typedef struct {
  *                own one suffix length (reads of one length of at most 255
  *                bases). */
 #define CXBWT_PLAN_DIGIT_LISTING 32
+/*  MERGE       - build reads of one length (at most 4096 bases) with the merge
+ *                plan (below) whatever the size, when the budget holds a
+ *                sort of the build in one slice; alone, or with ID64 (64-bit
+ *                rows). */
+#define CXBWT_PLAN_MERGE 64
 /* Test hook for failure handling: in the first digit pass of a build, tile 0
  * does not publish its counts, so tile 1's look-back wait runs out (after
  * wait_limit_ms).  The build then returns CXBWT_ETIMEOUT with unspecified
@@ -125,7 +130,14 @@ typedef struct {
 #define CXBWT_PLAN_TEST_STALL 4
 
 /* Sort plans.  Every plan computes the same B_R; they differ in speed only.
- *  AUTO     - GROUPS when the reads are at most 528 bases, else LSD.
+ *  AUTO     - for reads of one length in a build of one slice, when the
+ *             suffix list is not asked for and tile_items, prefix_len and
+ *             plan_flags are 0, the merge plan where it is the faster one (from
+ *             about 150,000 reads of 100 bases on): B_R built one suffix length
+ *             at a time, each step inserting the symbols before the suffixes
+ *             of that length, with no sort of the suffixes (the scheme of
+ *             Bauer, Cox & Rosone 2013).  Else GROUPS when the reads are at
+ *             most 528 bases, else LSD.
  *  LSD      - stable LSD radix passes over every 4-base digit of the
  *             A-padded suffixes (Section 3.2 as stated: one pass per digit).
  *  GROUPS   - LSD passes over the first l = 16 (or prefix_len = 12)
@@ -141,7 +153,7 @@ typedef struct {
   uint64_t bases;               /* sum of read lengths over those builds */
   uint64_t suffixes;            /* sum of N over those builds */
   uint64_t kernel_launches;     /* kernels this library launched */
-  uint64_t sort_pass_launches;  /* radix digit passes among them */
+  uint64_t sort_pass_launches;  /* radix digit passes among them (none in a build by the merge plan) */
   uint64_t sort_pass_items;     /* sum over digit passes of the items each one moved */
   double sort_pass_ms;          /* device time of the digit passes (only with `timing`) */
   double build_ms;              /* device time of whole builds (only with `timing`) */
@@ -157,7 +169,8 @@ typedef struct {
                                      previous pass carried, instead of generating ids or gathering it */
   uint64_t carried_pass_items;  /* sum over those passes of the items each one moved */
   double carried_pass_ms;       /* their device time, each pass between its own events (only with `timing`) */
-  uint64_t reserved[2];
+  uint64_t merge_launches;      /* steps of the merge plan (one per suffix length of a build that takes it) */
+  double merge_ms;              /* device time of the builds that took it (only with `timing`) */
 } cxbwt_stats;
 
 /* ABI version of the loaded library (CXBWT_ABI_VERSION it was built with). */

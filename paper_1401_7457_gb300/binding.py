@@ -46,7 +46,8 @@ class Stats(ctypes.Structure):
                 ("device_bytes_held", ctypes.c_uint64), ("group_ms", ctypes.c_double), ("emit_ms", ctypes.c_double),
                 ("slices", ctypes.c_uint64), ("cta_groups", ctypes.c_uint64), ("big_groups", ctypes.c_uint64),
                 ("carried_pass_launches", ctypes.c_uint64), ("carried_pass_items", ctypes.c_uint64),
-                ("carried_pass_ms", ctypes.c_double), ("reserved", ctypes.c_uint64 * 2)]
+                ("carried_pass_ms", ctypes.c_double), ("merge_launches", ctypes.c_uint64),
+                ("merge_ms", ctypes.c_double)]
 
     def as_dict(self):
         return {k: getattr(self, k) for k, _ in self._fields_ if k != "reserved"}
@@ -335,7 +336,7 @@ class Context:
 
     ALGO_AUTO, ALGO_LSD, ALGO_GROUPS = 0, 1, 2
     PLAN_ID64, PLAN_READ_MAJOR, PLAN_TEST_STALL, PLAN_CARRY_BASE, PLAN_NO_PREFETCH = 1, 2, 4, 8, 16
-    PLAN_DIGIT_LISTING = 32
+    PLAN_DIGIT_LISTING, PLAN_MERGE = 32, 64
 
     def __init__(self, device: int = 0, budget_bytes: int = 0, async_: bool = False, timing: bool = False,
                  tile_items: int = 0, algorithm: int = 0, plan_flags: int = 0, batch_workers: int = 0,

@@ -429,6 +429,107 @@ int split_pass(cxbwt_ctx* c, Run& r, const std::vector<Slice>& slices, const std
   return CXBWT_OK;
 }
 
+// Where a build's outputs go, and which of them are device memory.
+struct Outs {
+  uint32_t* bwt;
+  uint64_t *dollar, *counts, *sa;
+  bool bwt_dev, dollar_dev, counts_dev, sa_dev;
+};
+
+// The end of a build whose kernels and BWT copies are enqueued: the other
+// outputs' copies, the wait, the statistics (of n_sorted sorted slices: none
+// when the merge plan built it).
+static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_t n_sorted) {
+  const Plan& pl = r.pl;
+  cudaStream_t st = r.st;
+  const bool timing = c->opt.timing != 0;
+  if (timing) CX_CUDA(c, cudaEventRecord(c->ev[3], st));
+  if (!o.bwt_dev) {
+    CX_CUDA(c, cudaEventRecord(c->slice_done[0], c->side));
+    CX_CUDA(c, cudaStreamWaitEvent(st, c->slice_done[0], 0));
+  }
+  if (o.counts) {
+    CX_CUDA(c, cudaMemcpyAsync(o.counts, r.d_counts, 5 * 8, o.counts_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                               st));
+    if (!o.counts_dev) r.d2h += 40;
+  }
+  if (o.dollar && !o.dollar_dev) {
+    CX_CUDA(c, cudaMemcpyAsync(o.dollar, r.d_dollar, pl.n * 8, cudaMemcpyDeviceToHost, st));
+    r.d2h += pl.n * 8;
+  }
+  CX_CUDA(c, cudaMemcpyAsync(c->h_small + 4, r.d_err, 4, cudaMemcpyDeviceToHost, st));
+
+  c->stats.kernel_launches += r.launches + r.sort_launches;
+  c->stats.sort_pass_launches += r.sort_launches;
+  c->stats.sort_pass_items += r.sort_items;
+  c->stats.h2d_bytes += h2d;
+  c->stats.d2h_bytes += r.d2h;
+  c->stats.device_bytes_held = c->held;
+  c->stats.slices += std::max<size_t>(n_sorted, 1);
+  c->stats.carried_pass_launches += r.carried_launches;
+  c->stats.carried_pass_items += r.carried_items;
+  c->stats.merge_launches += r.merge_launches;
+
+  const bool host_out = !o.bwt_dev || (o.dollar && !o.dollar_dev) || (o.counts && !o.counts_dev) || (o.sa && !o.sa_dev);
+  if (c->opt.async && !host_out) {
+    // Completed (and checked) by cxbwt_sync.
+    c->stats.builds += 1;
+    c->stats.bases += pl.sum;
+    c->stats.suffixes += pl.N;
+    return CXBWT_OK;
+  }
+  CX_CUDA(c, cudaStreamSynchronize(st));
+  CX_TRY(take_device_error(c));
+  if (timing) {
+    float ms_all = 0;
+    CX_CUDA(c, cudaEventElapsedTime(&ms_all, c->ev[0], c->ev[3]));
+    for (size_t si = 0; si < n_sorted; ++si) {
+      cudaEvent_t* tev = &c->tev[4 * si];
+      float ms_sort = 0, ms_group = 0, ms_emit = 0;
+      CX_CUDA(c, cudaEventElapsedTime(&ms_sort, tev[0], tev[1]));
+      CX_CUDA(c, cudaEventElapsedTime(&ms_group, tev[1], tev[2]));
+      CX_CUDA(c, cudaEventElapsedTime(&ms_emit, tev[2], tev[3]));
+      c->stats.sort_pass_ms += ms_sort;
+      c->stats.group_ms += ms_group;
+      c->stats.emit_ms += ms_emit;
+    }
+    for (uint32_t j = 0; j < r.n_pev; ++j) {
+      if (!r.pev_carried[j]) continue;
+      float ms = 0;
+      CX_CUDA(c, cudaEventElapsedTime(&ms, c->pev[2 * size_t(j)], c->pev[2 * size_t(j) + 1]));
+      if (r.pev_carried[j] == 1) c->stats.carried_pass_ms += ms;
+      else c->stats.sort_pass_ms += ms;  // the split pass runs before every slice
+    }
+    c->stats.build_ms += ms_all;
+    if (!n_sorted) c->stats.merge_ms += ms_all;
+  }
+  c->stats.builds += 1;
+  c->stats.bases += pl.sum;
+  c->stats.suffixes += pl.N;
+  return CXBWT_OK;
+}
+
+// Whether the merge plan (merge.cu) is the faster one for a build, or a part
+// of `rows` of its rows, that a sort would make in one slice.  Fitted to both
+// plans' times with the store in L2 (reads x bases: merge against group plan):
+// 10k x 100 0.56 / 0.21 ms, 100k x 100 0.82 / 0.67, 300k x 100 1.26 / 1.63,
+// 1M x 36 0.84 / 1.62, 1M x 100 2.61 / 4.81, 250k x 400 8.00 / 8.25.  A merge
+// step costs 5.5 us and 11 + 0.115 L ps per read; the group plan 130 us and
+// 36 + 0.113 L ps per suffix, the LSD plan 6 ps per suffix and digit; a part
+// lists its rows among all suffixes (13 ps each) and sorts them.
+static bool merge_pays(const cxbwt_ctx* c, const Plan& pl, bool part, uint64_t rows) {
+  if (c->opt.algorithm != CXBWT_ALGO_AUTO || c->opt.tile_items || c->opt.prefix_len) return false;
+  if (c->opt.plan_flags & CXBWT_PLAN_MERGE) return (c->opt.plan_flags & ~(CXBWT_PLAN_MERGE | CXBWT_PLAN_ID64)) == 0;
+  if (c->opt.plan_flags) return false;
+  const double L = pl.Lmax, n = double(pl.n);
+  const double merge_us = (L + 1) * (5.5 + n * (11.0 + 0.115 * L) * 1e-6);
+  double sort_us = 130.0;
+  if (!pl.groups) sort_us += double(pl.N) * ((L + 3) / 4) * 6.0e-6;
+  else if (part) sort_us += double(pl.N) * 13.0e-6 + double(rows) * (20.0 + 0.113 * L) * 1e-6;
+  else sort_us += double(pl.N) * (36.0 + 0.113 * L) * 1e-6;
+  return merge_us < sort_us;
+}
+
 int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* lens, uint32_t* out_bwt,
                uint64_t* out_dollar, uint64_t* out_counts, uint64_t* out_sa, void* stream_v, const PartSpec* part) {
   if (!c) return CXBWT_EINVAL;
@@ -621,12 +722,17 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   uint64_t m1 = uint64_t(double(avail) / per_row);
   // A slice must fit 32-bit row counts; every workspace buffer below is
   // granted in 2 MB steps, so leave room for that rounding.
-  m1 = std::min<uint64_t>(m1 > (64u << 20) ? m1 - (1u << 20) : (m1 > 32768 ? m1 - 16384 : m1), 0xFFFFFFF0ull);
+  m1 = m1 > (64u << 20) ? m1 - (1u << 20) : (m1 > 32768 ? m1 - 16384 : m1);
+  const uint64_t m1_bytes = m1;  // by the budget alone (the merge plan has no limit of rows, when asked for)
+  m1 = std::min<uint64_t>(m1, 0xFFFFFFF0ull);
   std::vector<Slice> slices;
   uint64_t part_row0 = 0, part_rows = pl.N;  // global rows this call emits
   std::vector<uint32_t> P_host;  // per-position 4-mer counts, when the slices were planned from them
   bool refined = false;          // an 8-base bucket was split into 16-base ones
-  if (pl.N <= m1 && !part) {
+  // The merge plan sorts no slices.
+  bool merged = !out_sa && !part && merge_pays(c, pl, false, pl.N) &&
+                pl.N <= ((c->opt.plan_flags & CXBWT_PLAN_MERGE) ? m1_bytes : m1) && merge_fits(c, pl, out_more);
+  if ((pl.N <= m1 || merged) && !part) {
     Slice sl;
     sl.rows = uint32_t(pl.N);
     slices.push_back(sl);
@@ -787,11 +893,25 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     r.d_dollar = static_cast<uint64_t*>(c->out_dollar.p);
   }
 
-  if (slices.size() > 1 || part) {
-    CX_CUDA(c, cudaMemsetAsync(r.d_bwt, 0, bwt_words * 4, st));  // slice edges are merged with atomicOr
-  }
   if (part && r.d_dollar) {
     CX_CUDA(c, cudaMemsetAsync(r.d_dollar, 0xFF, n * 8, st));  // reads whose $ row is in another part
+  }
+
+  if (part && merge_pays(c, pl, true, part_rows) && pl.N <= m1 && merge_fits(c, pl, 0)) merged = true;
+  if (merged) {
+    if (part) CX_CUDA(c, cudaMemsetAsync(r.d_counts, 0, 5 * 8, st));
+    if (c->opt.timing) CX_CUDA(c, cudaEventRecord(c->ev[0], st));
+    CX_TRY(merge_run(c, r, part_row0, part_row0 + part_rows, word0, bwt_words, part != nullptr));
+    if (!bwt_dev && bwt_words) {
+      CX_CUDA(c, cudaMemcpyAsync(out_bwt, r.d_bwt, bwt_words * 4, cudaMemcpyDeviceToHost, st));
+      r.d2h += bwt_words * 4;
+    }
+    return finish_build(c, r, Outs{out_bwt, out_dollar, out_counts, out_sa, bwt_dev, dollar_dev, counts_dev, sa_dev}, h2d,
+                        0);
+  }
+
+  if (slices.size() > 1 || part) {
+    CX_CUDA(c, cudaMemsetAsync(r.d_bwt, 0, bwt_words * 4, st));  // slice edges are merged with atomicOr
   }
 
   uint32_t max_rows = 0;
@@ -928,68 +1048,8 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
       }
     }
   }
-  if (timing) CX_CUDA(c, cudaEventRecord(c->ev[3], st));
-  if (!bwt_dev) {
-    CX_CUDA(c, cudaEventRecord(c->slice_done[0], c->side));
-    CX_CUDA(c, cudaStreamWaitEvent(st, c->slice_done[0], 0));
-  }
-  if (out_counts) {
-    CX_CUDA(c, cudaMemcpyAsync(out_counts, r.d_counts, 5 * 8, counts_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                               st));
-    if (!counts_dev) r.d2h += 40;
-  }
-  if (out_dollar && !dollar_dev) {
-    CX_CUDA(c, cudaMemcpyAsync(out_dollar, r.d_dollar, n * 8, cudaMemcpyDeviceToHost, st));
-    r.d2h += n * 8;
-  }
-  CX_CUDA(c, cudaMemcpyAsync(c->h_small + 4, r.d_err, 4, cudaMemcpyDeviceToHost, st));
-
-  c->stats.kernel_launches += r.launches + r.sort_launches;
-  c->stats.sort_pass_launches += r.sort_launches;
-  c->stats.sort_pass_items += r.sort_items;
-  c->stats.h2d_bytes += h2d;
-  c->stats.d2h_bytes += r.d2h;
-  c->stats.device_bytes_held = c->held;
-  c->stats.slices += slices.size();
-  c->stats.carried_pass_launches += r.carried_launches;
-  c->stats.carried_pass_items += r.carried_items;
-
-  const bool host_out = !bwt_dev || (out_dollar && !dollar_dev) || (out_counts && !counts_dev) || (out_sa && !sa_dev);
-  if (c->opt.async && !host_out) {
-    // Completed (and checked) by cxbwt_sync.
-    c->stats.builds += 1;
-    c->stats.bases += pl.sum;
-    c->stats.suffixes += pl.N;
-    return CXBWT_OK;
-  }
-  CX_CUDA(c, cudaStreamSynchronize(st));
-  CX_TRY(take_device_error(c));
-  if (timing) {
-    float ms_all = 0;
-    CX_CUDA(c, cudaEventElapsedTime(&ms_all, c->ev[0], c->ev[3]));
-    for (size_t si = 0; si < slices.size(); ++si) {
-      cudaEvent_t* tev = &c->tev[4 * si];
-      float ms_sort = 0, ms_group = 0, ms_emit = 0;
-      CX_CUDA(c, cudaEventElapsedTime(&ms_sort, tev[0], tev[1]));
-      CX_CUDA(c, cudaEventElapsedTime(&ms_group, tev[1], tev[2]));
-      CX_CUDA(c, cudaEventElapsedTime(&ms_emit, tev[2], tev[3]));
-      c->stats.sort_pass_ms += ms_sort;
-      c->stats.group_ms += ms_group;
-      c->stats.emit_ms += ms_emit;
-    }
-    for (uint32_t j = 0; j < r.n_pev; ++j) {
-      if (!r.pev_carried[j]) continue;
-      float ms = 0;
-      CX_CUDA(c, cudaEventElapsedTime(&ms, c->pev[2 * size_t(j)], c->pev[2 * size_t(j) + 1]));
-      if (r.pev_carried[j] == 1) c->stats.carried_pass_ms += ms;
-      else c->stats.sort_pass_ms += ms;  // the split pass runs before every slice
-    }
-    c->stats.build_ms += ms_all;
-  }
-  c->stats.builds += 1;
-  c->stats.bases += pl.sum;
-  c->stats.suffixes += pl.N;
-  return CXBWT_OK;
+  return finish_build(c, r, Outs{out_bwt, out_dollar, out_counts, out_sa, bwt_dev, dollar_dev, counts_dev, sa_dev}, h2d,
+                      slices.size());
 }
 
 }  // namespace host
@@ -1126,7 +1186,7 @@ void cxbwt_destroy(cxbwt_ctx* c) {
   cudaDeviceSynchronize();
   DevBuf* bufs[] = {&c->vals[0], &c->vals[1], &c->keys[0], &c->keys[1], &c->status, &c->P, &c->base,
                     &c->lenhist, &c->desc, &c->misc, &c->store, &c->out_bwt, &c->out_dollar, &c->out_sa,
-                    &c->seglist, &c->rhist, &c->bhist};
+                    &c->seglist, &c->rhist, &c->bhist, &c->mstatus, &c->mtables};
   for (DevBuf* b : bufs) release(c, *b);
   for (auto& ev : c->ev)
     if (ev) cudaEventDestroy(ev);

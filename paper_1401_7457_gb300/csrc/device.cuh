@@ -165,4 +165,10 @@ __device__ __forceinline__ unsigned long long load_relaxed_u64(const unsigned lo
   return v;
 }
 
+// Asks the bulk-copy engine to bring `bytes` (a multiple of 16, 16-byte
+// aligned) of this GPU's memory into L2; nothing waits for it.
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 }  // namespace cxbwt

@@ -45,7 +45,7 @@ struct cxbwt_ctx {
   std::string err;
 
   DevBuf vals[2], keys[2], status, P, base, lenhist, desc, misc, store, out_bwt, out_dollar, out_sa, seglist, rhist,
-      bhist;
+      bhist, mstatus, mtables;
   uint32_t epoch = 0;
   cudaStream_t side = nullptr;            // device -> host streaming of finished slices
   cudaEvent_t slice_done[2] = {nullptr, nullptr};
@@ -245,6 +245,7 @@ struct Run {
   uint32_t bucket_bits = kBucketBits;  // slices are ranges of buckets of the first bucket_bits / 2 bases
   uint64_t launches = 0, sort_launches = 0, sort_items = 0, d2h = 0;
   uint64_t carried_launches = 0, carried_items = 0;
+  uint64_t merge_launches = 0;
   // Per-pass timing (timing option): pass j ran between events pev[2j] and
   // pev[2j+1]; pev_carried[j] says whether it was a carried-key pass.
   uint32_t n_pev = 0;
@@ -305,6 +306,14 @@ inline bool tuned_choice(const cxbwt_ctx* c, uint32_t max_len, uint64_t n_suffix
     }
   return false;
 }
+
+// Merge plan (merge.cu): whether a build of this plan's reads can take it
+// within the budget, `more` bytes aside; and all of its steps, writing rows [row_lo, row_hi) of
+// B_R as global words [word0, word0 + n_words) to r.d_bwt and their $ rows to
+// r.d_dollar, with the symbol counts of all of B_R, or of those rows alone
+// (count_rows, added to zeroed counts), in r.d_counts.
+bool merge_fits(const cxbwt_ctx* c, const Plan& pl, uint64_t more);
+int merge_run(cxbwt_ctx* c, Run& r, uint64_t row_lo, uint64_t row_hi, uint64_t word0, uint64_t n_words, bool count_rows);
 
 // Sort one slice into r.vals[*cur_out] (api.cu).
 int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t* tev);

@@ -48,10 +48,6 @@ __host__ __device__ constexpr uint32_t stage_ids_at(uint32_t rows) { return (row
 // Store words a tile stages: its reads' bases plus the word after them.
 constexpr uint32_t kListWords = kListMaxStage / 16 + 8;
 
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 // The first window of suffix (read at store offset off, position k) of a
 // read of L bases, A-padded, from the tile's store words sw (store word w_lo
 // at sw[0]); *prev = the base before it (0 when k = 0).  The same arithmetic

@@ -62,12 +62,6 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_256(uint32_t x, uint32_
   return warp_prefix + incl - x;
 }
 
-// Asks the bulk-copy engine to bring `bytes` (a multiple of 16, 16-byte
-// aligned) of this GPU's memory into L2; nothing waits for it.
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
 template <class V, int THREADS, int IPT, int MIN_BLOCKS, int MODE, bool WRITE_KEY, bool FILTER>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) k_onesweep(const PassArgs a) {
   constexpr int TILE = THREADS * IPT;
