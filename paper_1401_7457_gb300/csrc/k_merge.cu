@@ -275,37 +275,42 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
   constexpr uint32_t OLDP = OLD + OLD / 32 + 1;
   constexpr int WARPS = kMergeThreads / 32;
   constexpr int HELD = 2;                     // suffixes of the tile that a thread holds in registers
-  constexpr int AHEAD = 4;                    // loads in flight for the others
-  __shared__ __align__(16) uint32_t s_new[CH], s_lo[CH], s_hi[CH];  // rows inserted; their symbols, then the tile's planes
-  // The old planes (padded by a word per 32: a thread's reads start K words
-  // after its neighbour's), then, per class and chunk, the symbols (low half)
-  // and suffixes (high half) of the class in the tile's earlier chunks.
+  constexpr int AHEAD = 2;                    // loads in flight for the others
   constexpr uint32_t OLDW = (2 * OLDP + 3) / 4 * 4;
   constexpr uint32_t POOL = LAST ? OLDW : (4 * CH > OLDW ? 4 * CH : OLDW);
-  __shared__ __align__(16) uint32_t s_pool[POOL];
-  uint32_t* s_olo = s_pool;
-  uint32_t* s_ohi = s_pool + OLDP;
-  __shared__ uint32_t s_scan[WARPS];
-  __shared__ uint4 s_scan3[WARPS];
-  __shared__ uint4 s_item[WARPS];       // C, G, T suffixes before the tile, a part per warp
-  __shared__ Row s_old[3];              // C, G, T symbols of B_{j-1} before the tile's old rows
   // Per class: row in B_{j+1} of the tile's first symbol of it, the first row
   // of the second tile of B_{j+1} that it may reach, and its first suffix's
-  // place in the list; `two`: it does reach it.
+  // place in the list.
   struct Class {
     Row row, cross;
-    uint32_t at, two;
+    uint32_t at;
   };
-  __shared__ __align__(16) Class s_class[4];
-  __shared__ uint32_t s_cls[4 * 2 * 4]; // suffixes by class, first or second of those tiles, next symbol
+  struct __align__(16) Shared {
+    uint32_t fresh[CH], lo[CH], hi[CH];  // rows inserted; their symbols, then the tile's planes
+    // The old planes (padded by a word per 32: a thread's reads start K words
+    // after its neighbour's), then, per class and chunk, the symbols (low half)
+    // and suffixes (high half) of the class in the tile's earlier chunks.
+    uint32_t pool[POOL];
+    uint4 scan3[WARPS];
+    uint4 item[WARPS];                   // C, G, T suffixes before the tile, a share per warp
+    uint4 end;                           // low bits, high bits, both of the tile
+    uint32_t scan[WARPS];
+    uint32_t cls[4 * 2 * 4];             // suffixes by class, first or second of those tiles, next symbol
+    Row old[4];                          // C, G, T symbols of B_{j-1} before the tile's old rows
+    Row before[4];                       // C, G, T symbols of B_j before the tile
+    Class base[4];
+  };
+  __shared__ Shared sh;
+  uint32_t* const s_olo = sh.pool;
+  uint32_t* const s_ohi = sh.pool + OLDP;
 
-  const uint32_t lane = lane_id(), warp = __shfl_sync(0xFFFFFFFFu, threadIdx.x >> 5, 0), tid = warp * 32 + lane;
-  if (!LAST && tid < 32) s_cls[tid] = 0u;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (!LAST && tid < 32) sh.cls[tid] = 0u;
   {
     uint32_t z[K] = {};
-    reinterpret_cast<Vec*>(s_new)[tid] = W::make(z);
-    reinterpret_cast<Vec*>(s_lo)[tid] = W::make(z);
-    reinterpret_cast<Vec*>(s_hi)[tid] = W::make(z);
+    reinterpret_cast<Vec*>(sh.fresh)[tid] = W::make(z);
+    reinterpret_cast<Vec*>(sh.lo)[tid] = W::make(z);
+    reinterpret_cast<Vec*>(sh.hi)[tid] = W::make(z);
   }
   __syncthreads();         // the tile's words are zeroed
   grid_dependency_wait();  // the step before wrote what is read from here on
@@ -376,37 +381,23 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
     old_h = __ldcg(hi4 + tid);
   }
   if (!LAST && warp == WARPS - 1) {
-    // Symbols of B_{j-1} before row o0: before its tile, before the part of
-    // the tile that one warp wrote, and in that part (at most 128 words).
-    const uint32_t u = uint32_t(o0 >> a.prev_shift), in = uint32_t(o0) & ((1u << a.prev_shift) - 1);
-    const uint32_t part_shift = a.prev_shift - 3, part = in >> part_shift, rest = in & ((1u << part_shift) - 1);
+    // Symbols of B_{j-1} before row o0: before its tile, before its part of
+    // the tile, and in the part (a word per lane).
+    const uint32_t u = uint32_t(o0 >> a.prev_shift), part = (uint32_t(o0) & ((1u << a.prev_shift) - 1)) / kMergePart;
+    const uint32_t rest = uint32_t(o0) % kMergePart;
     uint64_t whole = 0, parts = 0;
     if (a.step && lane < 3) {
       whole = __ldcg(a.before_in + 4 * uint64_t(u) + lane);
-      if (part) parts = __ldcg(a.parts_in + 8 * uint64_t(u) + part);
+      if (part) parts = __ldcg(a.parts_in + (uint64_t(u) << (a.prev_shift - 10)) + part);
     }
-    const uint32_t w0 = uint32_t((o0 - rest) >> 5);
-    uint32_t l[4], h[4];
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const uint32_t at = 32 * x + lane;
-      const bool some = 32 * at < rest;
-      l[x] = some ? __ldcg(a.lo_in + w0 + at) : 0u;
-      h[x] = some ? __ldcg(a.hi_in + w0 + at) : 0u;
-    }
-    uint32_t nc = 0, ng = 0, nt_ = 0;
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const uint32_t at = 32 * (32 * x + lane);
-      const uint32_t keep = rest >= at + 32 ? 0xFFFFFFFFu : rest > at ? (1u << (rest - at)) - 1 : 0u;
-      nc += __popc(l[x] & ~h[x] & keep);
-      ng += __popc(h[x] & ~l[x] & keep);
-      nt_ += __popc(l[x] & h[x] & keep);
-    }
+    const uint32_t at = uint32_t((o0 - rest) >> 5) + lane;
+    const uint32_t keep = rest >= 32 * lane + 32 ? 0xFFFFFFFFu : rest > 32 * lane ? (1u << (rest - 32 * lane)) - 1 : 0u;
+    const uint32_t l = keep ? __ldcg(a.lo_in + at) & keep : 0u, h = keep ? __ldcg(a.hi_in + at) & keep : 0u;
+    uint32_t nc = __popc(l & ~h), ng = __popc(h & ~l), nt_ = __popc(l & h);
     nc = __reduce_add_sync(0xFFFFFFFFu, nc);
     ng = __reduce_add_sync(0xFFFFFFFFu, ng);
     nt_ = __reduce_add_sync(0xFFFFFFFFu, nt_);
-    if (lane < 3) s_old[lane] = Row(whole) + (uint32_t(parts >> (16 * lane)) & 0xFFFFu) + (lane == 0 ? nc : lane == 1 ? ng : nt_);
+    if (lane < 3) sh.old[lane] = Row(whole) + (uint32_t(parts >> (16 * lane)) & 0xFFFFu) + (lane == 0 ? nc : lane == 1 ? ng : nt_);
   }
   if (!LAST) {
     uint32_t c = in_group.x + (uint32_t(in_tile) & 0xFFFFu), g = in_group.y + (uint32_t(in_tile >> 16) & 0xFFFFu),
@@ -420,7 +411,7 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
     c = __reduce_add_sync(0xFFFFFFFFu, c);
     g = __reduce_add_sync(0xFFFFFFFFu, g);
     t = __reduce_add_sync(0xFFFFFFFFu, t);
-    if (lane == 0) s_item[warp] = make_uint4(c, g, t, 0u);
+    if (lane == 0) sh.item[warp] = make_uint4(c, g, t, 0u);
   }
   {
     auto keep_old = [&](uint32_t x, const uint4& l, const uint4& h) {
@@ -453,14 +444,14 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
       return;
     }
     const uint32_t bit = 1u << (r & 31);
-    or_shared_if(s_new + (r >> 5), bit, 1u);
+    or_shared_if(sh.fresh + (r >> 5), bit, 1u);
     if (LAST) {
       // The suffix is the whole read: $ (code 0) precedes it.
       const uint64_t p = uint64_t(t0) + r;
       if (a.dollar_pos && read < a.n && p >= a.row_lo && p < a.row_hi) a.dollar_pos[read] = p;
     } else {
-      or_shared_if(s_lo + (r >> 5), bit, w & 1);
-      or_shared_if(s_hi + (r >> 5), bit, w & 2);
+      or_shared_if(sh.lo + (r >> 5), bit, w & 1);
+      or_shared_if(sh.hi + (r >> 5), bit, w & 2);
     }
   };
 #pragma unroll
@@ -496,19 +487,39 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
 
   // ---- the new rows before each thread's first chunk ---------------------------
   uint32_t mm[K], lo[K], hi[K];
-  W::get(reinterpret_cast<const Vec*>(s_new)[tid], mm);
+  W::get(reinterpret_cast<const Vec*>(sh.fresh)[tid], mm);
   uint32_t cnt = 0;
 #pragma unroll
   for (int k = 0; k < K; ++k) cnt += __popc(mm[k]);
   uint32_t before = cnt;
   warp_scan(before);
-  if (lane == 31) s_scan[warp] = before;
+  if (lane == 31) sh.scan[warp] = before;
   __syncthreads();
-  before += sum_before(s_scan[lane & (WARPS - 1)], lane, warp) - cnt;
+  before += sum_before(sh.scan[lane & (WARPS - 1)], lane, warp) - cnt;
+
+  if (!LAST && warp == WARPS - 1) {
+    // Lane c: class c's symbols and suffixes before the tile.
+    const uint4 it = sh.item[lane & (WARPS - 1)];
+    const uint32_t ic = __reduce_add_sync(0xFFFFFFFFu, lane < WARPS ? it.x : 0u), ig = __reduce_add_sync(0xFFFFFFFFu, lane < WARPS ? it.y : 0u),
+                   itt = __reduce_add_sync(0xFFFFFFFFu, lane < WARPS ? it.z : 0u);
+    const Row bc = sh.old[0] + ic, bg = sh.old[1] + ig, bt = sh.old[2] + itt;  // symbols of B_j before the tile
+    if (lane < 3) {
+      const Row b = lane == 0 ? bc : lane == 1 ? bg : bt;
+      sh.before[lane] = b;
+      a.before_out[4 * uint64_t(tile) + lane] = b;
+    }
+    if (lane < 4) {
+      const Row row = row_base + (lane == 0 ? t0 - bc - bg - bt : lane == 1 ? bc : lane == 2 ? bg : bt);
+      const uint32_t at = item_base + (lane == 0 ? s0 - ic - ig - itt : lane == 1 ? ic : lane == 2 ? ig : itt);
+      // Tiles of B_{j+1} are at least as large as this one: the class's
+      // symbols, consecutive rows there, reach two at most.
+      sh.base[lane] = Class{row, Row((row >> a.next_shift) + 1) << a.next_shift, at};
+    }
+  }
 
   // ---- merge: old symbols spread around the new rows ---------------------------
-  W::get(reinterpret_cast<const Vec*>(s_lo)[tid], lo);
-  W::get(reinterpret_cast<const Vec*>(s_hi)[tid], hi);
+  W::get(reinterpret_cast<const Vec*>(sh.lo)[tid], lo);
+  W::get(reinterpret_cast<const Vec*>(sh.hi)[tid], hi);
   const uint32_t o_first = skip + 32 * K * tid - before;  // old row, from row 32 * c0 on
   uint32_t xl[K], xh[K];                                  // per chunk, the next 32 old symbols
   if (K == 1 || !__any_sync(0xFFFFFFFFu, cnt > 32)) {
@@ -626,54 +637,35 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
   }
   uint32_t i0 = tl, i1 = th, i2 = tt;
   warp_scan(i0, i1, i2);
-  if (lane == 31) s_scan3[warp] = make_uint4(i0, i1, i2, 0u);
+  if (lane == 31) sh.scan3[warp] = make_uint4(i0, i1, i2, 0u);
   {
     // Planes out: whole tiles (the arrays hold whole tiles; rows past the end are 0).
     const uint64_t at = uint64_t(tile) * kMergeThreads + tid;
     __stcg(reinterpret_cast<Vec*>(a.lo_out) + at, W::make(lo));
     __stcg(reinterpret_cast<Vec*>(a.hi_out) + at, W::make(hi));
-    reinterpret_cast<Vec*>(s_lo)[tid] = W::make(lo);
-    reinterpret_cast<Vec*>(s_hi)[tid] = W::make(hi);
+    reinterpret_cast<Vec*>(sh.lo)[tid] = W::make(lo);
+    reinterpret_cast<Vec*>(sh.hi)[tid] = W::make(hi);
   }
   __syncthreads();
   {
-    const uint4 x = s_scan3[lane & (WARPS - 1)];
+    const uint4 x = sh.scan3[lane & (WARPS - 1)];
     i0 += sum_before(x.x, lane, warp);
     i1 += sum_before(x.y, lane, warp);
     i2 += sum_before(x.z, lane, warp);
   }
-  if (lane == 0) {
-    // Symbols before the warp's rows in the tile, for the next step.
+  if (tid == kMergeThreads - 1) sh.end = make_uint4(i0, i1, i2, 0u);
+  if (lane % (32 / K) == 0) {
+    // Symbols before the part that starts with the lane's rows, for the next step.
     const uint32_t l = i0 - tl, h = i1 - th, t = i2 - tt;
-    a.parts_out[8 * uint64_t(tile) + warp] =
+    a.parts_out[(CH * uint64_t(tile) + K * tid) / 32] =
         (uint64_t(t & 0xFFFFu) << 32) | (uint64_t((h - t) & 0xFFFFu) << 16) | ((l - t) & 0xFFFFu);
   }
-  if (warp == WARPS - 1) {
-    // Lane c: class c's symbols and suffixes before the tile, and in it.
-    const uint32_t e0 = __shfl_sync(0xFFFFFFFFu, i0, 31), e1 = __shfl_sync(0xFFFFFFFFu, i1, 31), e2 = __shfl_sync(0xFFFFFFFFu, i2, 31);
-    const uint4 it = s_item[lane & (WARPS - 1)];
-    const uint32_t ic = __reduce_add_sync(0xFFFFFFFFu, lane < WARPS ? it.x : 0u), ig = __reduce_add_sync(0xFFFFFFFFu, lane < WARPS ? it.y : 0u),
-                   itt = __reduce_add_sync(0xFFFFFFFFu, lane < WARPS ? it.z : 0u);
-    const Row bc = s_old[0] + ic, bg = s_old[1] + ig, bt = s_old[2] + itt;  // symbols of B_j before the tile
-    const uint32_t C = (e0 - e2) & 0xFFFFu, G = (e1 - e2) & 0xFFFFu, T = e2 & 0xFFFFu;
-    if (lane < 3) {
-      const Row b = lane == 0 ? bc : lane == 1 ? bg : bt;
-      a.before_out[4 * uint64_t(tile) + lane] = b;
-      if (tile == a.n_tiles - 1) a.before_out[4 * uint64_t(tile + 1) + lane] = b + (lane == 0 ? C : lane == 1 ? G : T);
-    }
-    if (lane < 4) {
-      const Row rc = lane == 0 ? t0 - bc - bg - bt : lane == 1 ? bc : lane == 2 ? bg : bt;
-      const uint32_t first = lane == 0 ? s0 - ic - ig - itt : lane == 1 ? ic : lane == 2 ? ig : itt;
-      const uint32_t total = lane == 0 ? rows - C - G - T : lane == 1 ? C : lane == 2 ? G : T;
-      const Row row = row_base + rc;
-      const uint32_t at = item_base + first;
-      // Tiles of B_{j+1} are at least as large as this one: the class's
-      // symbols, consecutive rows there, reach two at most.
-      const Row next = Row((row >> a.next_shift) + 1) << a.next_shift;
-      s_class[lane] = Class{row, next, at, row + total > next ? 1u : 0u};
-      if (total && (row & ((Row(1) << a.next_shift) - 1)) == 0 && (row >> a.next_shift) < a.next_tiles)
-        a.start_out[row >> a.next_shift] = at;
-    }
+  if (tile == a.n_tiles - 1 && tid == kMergeThreads - 1) {
+    // Symbols in all of B_j.
+    unsigned long long* end = reinterpret_cast<unsigned long long*>(a.before_out) + 4 * uint64_t(tile + 1);
+    end[0] = sh.before[0] + ((i0 - i2) & 0xFFFFu);
+    end[1] = sh.before[1] + ((i1 - i2) & 0xFFFFu);
+    end[2] = sh.before[2] + (i2 & 0xFFFFu);
   }
   // (the old planes were last read before the barrier above)
   {
@@ -689,7 +681,7 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
       q[3][k] = t;
       news += __popc(mm[k]);
     }
-    auto* pool = reinterpret_cast<Vec*>(s_pool);
+    auto* pool = reinterpret_cast<Vec*>(sh.pool);
 #pragma unroll
     for (int c = 0; c < 4; ++c) pool[c * kMergeThreads + tid] = W::make(q[c]);
   }
@@ -700,15 +692,15 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
   auto place = [&](uint32_t r, uint32_t read, uint32_t w) {
     if (r >= rows) return;
     const uint32_t q = r >> 5, c = w & 3;
-    const Class base = s_class[c];
+    const Class base = sh.base[c];
     // Rows of symbol c below r in its chunk.
-    const uint32_t same = (s_lo[q] ^ ((c & 1) - 1)) & (s_hi[q] ^ ((c >> 1) - 1)) & ((1u << (r & 31)) - 1);
-    const uint32_t counts = s_pool[c * CH + q];
+    const uint32_t same = (sh.lo[q] ^ ((c & 1) - 1)) & (sh.hi[q] ^ ((c >> 1) - 1)) & ((1u << (r & 31)) - 1);
+    const uint32_t counts = sh.pool[c * CH + q];
     const Row row = base.row + ((counts & 0xFFFFu) + __popc(same));
-    const uint32_t at = base.at + (counts >> 16) + __popc(same & s_new[q]);
+    const uint32_t at = base.at + (counts >> 16) + __popc(same & sh.fresh[q]);
     w >>= 2;
     if (a.refill) w = bases_before(a.R, uint64_t(min(read, a.n - 1)) * a.R.uniform_len, a.R.uniform_len - (a.step + 1));
-    atomicAdd(&s_cls[c * 8 + (row >= base.cross ? 4u : 0u) + (w & 3)], 1u);
+    atomicAdd(&sh.cls[c * 8 + (row >= base.cross ? 4u : 0u) + (w & 3)], 1u);
     if (at < a.n) {
       __stcg(a.key_out + at, WIDE ? (uint64_t(read) << a.pshift) | (uint64_t(row) & pmask) : (uint64_t(read) << 32) | row);
       __stcg(a.bases_out + at, w);
@@ -740,12 +732,16 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
   // ---- suffixes in and before the tiles of B_{j+1} -----------------------------------
   if (tid < 8) {
     const uint32_t c = tid >> 1, second = tid & 1;
-    const uint32_t* n_cls = s_cls + tid * 4;
-    const Class base = s_class[c];
+    const uint32_t* n_cls = sh.cls + tid * 4;
+    const Class base = sh.base[c];
+    const uint32_t e0 = sh.end.x, e1 = sh.end.y, e2 = sh.end.z;
+    const uint32_t C = (e0 - e2) & 0xFFFFu, G = (e1 - e2) & 0xFFFFu, T = e2 & 0xFFFFu;
+    const uint32_t total = c == 0 ? rows - C - G - T : c == 1 ? C : c == 2 ? G : T;
     const uint32_t to = uint32_t(base.cross >> a.next_shift) - 1 + second;
-    if (second && base.two && to < a.next_tiles) {
+    const Row first = second ? base.cross : Row(base.cross - (Row(1) << a.next_shift));  // of tile `to`
+    if (first >= base.row && first < base.row + total && to < a.next_tiles) {
       const uint32_t* n_first = n_cls - 4;
-      a.start_out[to] = base.at + n_first[0] + n_first[1] + n_first[2] + n_first[3];
+      a.start_out[to] = base.at + (second ? n_first[0] + n_first[1] + n_first[2] + n_first[3] : 0u);
     }
     if (to < a.next_tiles) add_class_counts(a.tiles_out, a.groups_out, to, n_cls[1], n_cls[2], n_cls[3]);
   }

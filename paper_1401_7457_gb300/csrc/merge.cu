@@ -59,7 +59,7 @@ Layout layout_of(const cxbwt_ctx* c, const Plan& pl) {
   auto pad = [](uint64_t x) { return (x + 255) / 256 * 256; };
   z.starts = pad((tiles + 2) * 4);
   z.before = pad((tiles + 2) * 32);
-  z.parts = pad((tiles + 2) * 64);
+  z.parts = pad((pl.N / kMergePart + 2 * kMergeMaxTile / kMergePart) * 8);
   z.tiles = pad((tiles + 2) * 8);
   z.groups = pad((tiles / kMergeGroupTiles + 2) * 16);
   // Starts, tile counts and group counts must be zero at first: side by side.

@@ -13,6 +13,7 @@ constexpr uint32_t kMergeBlocks = 5;      // CTAs per SM the registers are sized
 constexpr uint32_t merge_tile_rows(uint32_t k) { return kMergeThreads * 32u * k; }
 constexpr uint32_t merge_tile_shift(uint32_t k) { return k == 1 ? 13u : k == 2 ? 14u : 15u; }
 constexpr uint32_t kMergeMaxTile = merge_tile_rows(4);
+constexpr uint32_t kMergePart = 1024;     // rows whose counts are kept from one step to the next
 constexpr uint32_t kMergeMaxLen = 4096;   // reads the tables below are built for
 constexpr uint32_t kMergeGroupTiles = 256;  // tiles whose counts are also summed together
 
@@ -43,8 +44,8 @@ struct MergeArgs {
   uint32_t pshift;
   const uint64_t* row_base;    // [4] first row of B_{j+1} of each class (suffixes starting with A, C, G, T)
   const uint32_t* item_base;   // [4] first suffix of length j + 1 of each class
-  // Symbols C, G, T (as 64-bit counts; 4 words per tile) before each tile,
-  // and (three 16-bit counts; 8 words per tile) before each warp's rows in it.
+  // Symbols C, G, T (as 64-bit counts; 4 words per tile) before each tile, and
+  // (three 16-bit counts) before each part of kMergePart rows in its tile.
   uint32_t prev_shift;               // tiles of B_{j-1} have 2^prev_shift rows (at most B_j's)
   const uint64_t* before_in;
   const uint64_t* parts_in;
