@@ -1027,7 +1027,7 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     e.read_base = 0;
     e.n_reads_out = uint32_t(n);
     CX_CUDA(c, launch_emit(e, st));
-    ++r.launches;
+    r.launches += e.sa_out ? 2 : 1;
     if (tev) CX_CUDA(c, cudaEventRecord(tev[3], st));
     if (out_sa && !sa_dev) {
       CX_CUDA(c, cudaMemcpyAsync(out_sa + sl.row0, r.d_sa, uint64_t(sl.rows) * 8, cudaMemcpyDeviceToHost, st));

@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(const EmitArgs a) {
           cpack += 1ull << (8 * (sym + 1));
         }
         word |= sym << (30 - 2 * j);
-        if (a.sa_out) a.sa_out[g - a.row0] = (uint64_t(s.read - a.read_base) << 16) | s.k;
       }
     }
     if (whole) a.bwt[w - a.word_base] = word;
@@ -98,12 +97,40 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(const EmitArgs a) {
   if (threadIdx.x < 5 && s_cnt[threadIdx.x]) atomicAdd(a.counts + threadIdx.x, s_cnt[threadIdx.x]);
 }
 
+// The sorted suffix list, (read << 16) | offset per row: a kernel of its own,
+// whose threads take consecutive rows.  Written by the threads above, 16 rows
+// each, every store of a warp touched 32 sectors (60M rows: emission 638 us,
+// against 224 and 100 us apart).
+template <class V>
+__global__ void __launch_bounds__(kEmitThreads) k_emit_sa(const EmitArgs a) {
+  constexpr int kRows = 4;
+  const V* sa = static_cast<const V*>(a.sa);
+  const uint64_t r0 = uint64_t(blockIdx.x) * (kEmitThreads * kRows) + threadIdx.x;
+  V v[kRows];
+#pragma unroll
+  for (int j = 0; j < kRows; ++j) v[j] = r0 + j * kEmitThreads < a.n ? __ldg(sa + r0 + j * kEmitThreads) : V(0);
+#pragma unroll
+  for (int j = 0; j < kRows; ++j) {
+    const uint64_t r = r0 + j * kEmitThreads;
+    if (r >= a.n) break;
+    const uint32_t read = uint32_t(v[j] >> a.R.shift), k = (uint32_t(v[j]) & ((1u << a.R.shift) - 1u)) >> a.R.sym_bits;
+    a.sa_out[r] = (uint64_t(read - a.read_base) << 16) | k;
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_emit(const EmitArgs& a, cudaStream_t st) {
   if (a.n == 0) return cudaSuccess;
   const uint64_t words = ((a.row0 + a.n + 15) >> 4) - (a.row0 >> 4);
   const uint64_t blocks = (words + kEmitThreads - 1) / kEmitThreads;
+  if (a.sa_out) {
+    const uint64_t sa_blocks = (uint64_t(a.n) + kEmitThreads * 4 - 1) / (kEmitThreads * 4);
+    if (a.id_bytes == 8) k_emit_sa<uint64_t><<<uint32_t(sa_blocks), kEmitThreads, 0, st>>>(a);
+    else k_emit_sa<uint32_t><<<uint32_t(sa_blocks), kEmitThreads, 0, st>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   if (a.id_bytes == 8) k_emit<uint64_t><<<uint32_t(blocks), kEmitThreads, 0, st>>>(a);
   else k_emit<uint32_t><<<uint32_t(blocks), kEmitThreads, 0, st>>>(a);
   return cudaGetLastError();
