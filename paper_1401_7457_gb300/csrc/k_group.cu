@@ -546,6 +546,7 @@ cudaError_t launch_v(const SegArgs& a, int nw, int sm_count, bool wide, cudaStre
     case 10: return launch_nw<10, V>(a, sm_count, wide, st);
     case 12: return launch_nw<12, V>(a, sm_count, wide, st);
     case 16: return launch_nw<16, V>(a, sm_count, wide, st);
+    case 20: return launch_nw<20, V>(a, sm_count, wide, st);
     case 24: return launch_nw<24, V>(a, sm_count, wide, st);
     case 32: return launch_nw<32, V>(a, sm_count, wide, st);
     default: return cudaErrorInvalidValue;
@@ -564,6 +565,7 @@ int segsort_words(uint32_t max_len, uint32_t depth) {
   if (nw <= 10) return 10;
   if (nw <= 12) return 12;
   if (nw <= 16) return 16;
+  if (nw <= 20) return 20;  // (reads of 300 bases: 2,094 us, 2,418 with 24 words)
   if (nw <= 24) return 24;
   if (nw <= 32) return 32;
   return 0;  // reads too long for the on-chip finish
