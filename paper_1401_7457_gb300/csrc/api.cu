@@ -79,6 +79,11 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
   // whole: rows 0..d_sorted-1 = char digits d, rows D.. = length digits.
   // slice: row 0 = suffix length (its low byte), rows 1..4 = window-0 digits
   // (most significant first), row 5 = the high byte of the suffix length.
+  // A slice of whole 4-base buckets listed by the listing kernel: its digits
+  // are counted from the listed keys (4 bytes each) instead of by a scan of
+  // every suffix of the collection (505M suffixes in three slices: 1.52 ms a
+  // slice, against 0.25 ms for its 168M keys).
+  const bool count_listed = r.P_host && !sl.whole && !sl.pregen && pl.uniform && r.read_major && list_kernel(c, pl);
   if (sl.pregen) {
     // The slice's first windows are listed already: count their digits (rows 1..4).
     CX_CUDA(c, cudaMemsetAsync(r.base + kRadix, 0, 4 * kRadix * 4, st));
@@ -90,6 +95,20 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
     CX_CUDA(c, launch_digitbase(static_cast<const uint32_t*>(c->P.p), pl.Lmax, d_sorted, pl.uniform ? 1 : 0,
                                 uint32_t(pl.n), pl.Lmax, static_cast<const uint32_t*>(c->lenhist.p), r.base, st));
     r.launches += 2;
+  } else if (count_listed) {
+    // Suffixes per length of the slice's 4-base buckets: of length t, those
+    // whose 4-mer at position L - t is in the slice; the terminator-only ones
+    // are in bucket 0.  The window digits are counted once the slice is listed.
+    std::vector<uint32_t> first(kRadix, 0);
+    uint64_t acc = 0;
+    for (uint32_t t = 0; t <= pl.Lmax; ++t) {
+      first[t] = uint32_t(acc);
+      for (uint64_t b = sl.key_lo >> 24; b < (sl.key_hi >> 24); ++b)
+        acc += t ? (*r.P_host)[size_t(pl.Lmax - t) * kRadix + b] : (b ? 0 : pl.n);
+    }
+    if (acc != sl.rows)
+      return fail(c, CXBWT_EINTERNAL, "a slice of %u suffixes, %llu by length", sl.rows, (unsigned long long)acc);
+    CX_CUDA(c, cudaMemcpyAsync(r.base, first.data(), kRadix * 4, cudaMemcpyHostToDevice, st));
   } else {
     CX_CUDA(c, cudaMemsetAsync(r.base, 0, 6 * kRadix * 4, st));
     CX_CUDA(c, launch_pass_hist(r.R, uint32_t(pl.n), sl.key_lo, uint32_t(sl.key_hi - 1 - sl.key_lo), r.base,
@@ -192,6 +211,11 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
     if (tev) CX_TRY(pass_event_begin(c, r));
     CX_CUDA(c, launch_list(la, idb, st));
     if (tev) CX_TRY(pass_event_end(c, r, 0));
+    if (count_listed) {
+      CX_CUDA(c, cudaMemsetAsync(r.base + kRadix, 0, 4 * kRadix * 4, st));
+      CX_CUDA(c, launch_key_hist(r.keys[kin], sl.rows, r.base + kRadix, c->sm_count, st));
+      r.launches += 2;
+    }
     cur ^= 1;
     ++r.sort_launches;
     r.sort_items += sl.rows;
@@ -869,6 +893,7 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
       for (uint32_t b = b_hi; b < bh.size(); ++b) total += bh[b];
       if (total != pl.N) return fail(c, CXBWT_EINTERNAL, "bucket counts sum to %llu, not N", (unsigned long long)total);
     }
+    if (!part && r.bucket_bits == 8 && !refined) r.P_host = &P_host;
     // Gathers walk the store in address order when it is too big for L2.
     r.read_major = pl.Lmax <= 255 && (pl.n_words * 4 > (64u << 20) || (c->opt.plan_flags & CXBWT_PLAN_READ_MAJOR));
   }

@@ -242,6 +242,7 @@ struct Run {
   uint64_t* d_dollar = nullptr;
   uint64_t* d_sa = nullptr;       // global rows
   bool read_major = false;        // multi-slice first pass in read-major order
+  const std::vector<uint32_t>* P_host = nullptr;  // per-position 4-mer counts, when the slices are whole 4-base buckets
   uint32_t bucket_bits = kBucketBits;  // slices are ranges of buckets of the first bucket_bits / 2 bases
   uint64_t launches = 0, sort_launches = 0, sort_items = 0, d2h = 0;
   uint64_t carried_launches = 0, carried_items = 0;
