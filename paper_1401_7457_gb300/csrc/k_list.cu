@@ -48,41 +48,31 @@ __host__ __device__ constexpr uint32_t stage_ids_at(uint32_t rows) { return (row
 // Store words a tile stages: its reads' bases plus the word after them.
 constexpr uint32_t kListWords = kListMaxStage / 16 + 8;
 
-// The first window of suffix (read at store offset off, position k) of a
-// read of L bases, A-padded, from the tile's store words sw (store word w_lo
-// at sw[0]); *prev = the base before it (0 when k = 0).  The same arithmetic
-// as window16_pair_prev, on shared memory.
-__device__ __forceinline__ uint32_t window_staged(const uint32_t* sw, uint64_t w_lo, uint64_t off, uint32_t k,
-                                                  uint32_t L, uint32_t* prev) {
-  const bool inside = k < L;
-  const uint32_t rem = inside ? L - k : 0u;
-  const uint64_t q = off + (inside ? k : 0u);
-  const uint32_t w = uint32_t((q >> 4) - w_lo);
-  const uint32_t sh = uint32_t(q & 15u) * 2u;
+// The 16 bases from the tile's staged base q on (q counted from its first
+// store word), those past the read's end masked away by `keep`; *prev = the
+// base before q (read only when `has_prev`).
+__device__ __forceinline__ uint32_t window_staged(const uint32_t* sw, uint32_t q, uint32_t keep, bool has_prev, uint32_t* prev) {
+  const uint32_t w = q >> 4, sh = (q & 15u) * 2u;
   const uint32_t w0 = sw[w];
-  const uint32_t key = __funnelshift_l(sw[w + 1], w0, sh);
-  const uint32_t keep = rem >= 16u ? 0xFFFFFFFFu : ~(0xFFFFFFFFu >> (2u * rem));
+  const uint32_t key = __funnelshift_l(sw[w + 1], w0, sh) & keep;
   if (prev) {
-    uint32_t p = 0;
-    if (k != 0) {
-      const uint64_t qp = off + k - 1;
-      const uint32_t wp = uint32_t((qp >> 4) - w_lo);
-      p = ((wp == w ? w0 : sw[wp]) >> (30u - 2u * uint32_t(qp & 15u))) & 3u;
-    }
-    *prev = p;
+    const uint32_t qp = q - 1;
+    *prev = has_prev ? ((sh ? w0 : sw[qp >> 4]) >> (30u - 2u * (qp & 15u))) & 3u : 0u;
   }
-  return key & keep;
+  return key;
 }
 
+// NS: key ranges compiled in (1, or up to kMaxSplit of which n_slices are used).
+template <int NS>
 __device__ __forceinline__ uint32_t slice_of(const ListArgs& a, uint32_t key) {
-  uint32_t s = kMaxSplit;
+  uint32_t s = NS;
 #pragma unroll
-  for (int j = kMaxSplit - 1; j >= 0; --j)
-    if (uint32_t(j) < a.n_slices && key - a.key_lo[j] <= a.key_last[j]) s = uint32_t(j);
+  for (int j = NS - 1; j >= 0; --j)
+    if ((NS == 1 || uint32_t(j) < a.n_slices) && key - a.key_lo[j] <= a.key_last[j]) s = uint32_t(j);
   return s;
 }
 
-template <class V, int THREADS>
+template <class V, int THREADS, int NS>
 __global__ void __launch_bounds__(THREADS) k_list(const ListArgs a) {
   constexpr int WARPS = THREADS / 32;
   constexpr int PER = kSlots / THREADS;  // slots per thread in the scan and the look-back
@@ -137,19 +127,34 @@ __global__ void __launch_bounds__(THREADS) k_list(const ListArgs a) {
   __syncthreads();
 
   // ---- 1. count ------------------------------------------------------------------
-  uint32_t cnt[kMaxSplit];
+  // Thread k's windows start L bases apart: 32-bit positions from the tile's
+  // first store word on, one addition per read.  With one key range the reads
+  // it keeps are also noted, a bit each (the first 64), so that the second walk
+  // takes those alone (505M suffixes, a third kept: 3.41 -> 2.41 ms).
+  uint32_t cnt[NS];
 #pragma unroll
-  for (int s = 0; s < kMaxSplit; ++s) cnt[s] = 0u;
+  for (int s = 0; s < NS; ++s) cnt[s] = 0u;
+  const uint32_t rem = L - min(k, L);
+  const uint32_t keep = rem >= 16u ? 0xFFFFFFFFu : ~(0xFFFFFFFFu >> (2u * rem));
+  const uint32_t q0 = uint32_t(uint64_t(ra) * L - (w_lo << 4)) + (k < L ? k : 0u);
+  unsigned long long kept = 0;
   if (act) {
-    for (uint32_t i = ra; i < rb; ++i) {
-      const uint32_t s = slice_of(a, window_staged(s_words, w_lo, uint64_t(i) * L, k, L, nullptr));
+    uint32_t q = q0;
+    for (uint32_t i = ra; i < rb; ++i, q += L) {
+      const uint32_t s = slice_of<NS>(a, window_staged(s_words, q, keep, false, nullptr));
+      if (NS == 1) {
+        const uint32_t on = s == 0u ? 1u : 0u;
+        cnt[0] += on;
+        if (i - ra < 64u) kept |= (unsigned long long)on << (i - ra);
+      } else {
 #pragma unroll
-      for (int j = 0; j < kMaxSplit; ++j) cnt[j] += (s == uint32_t(j)) ? 1u : 0u;
+        for (int j = 0; j < NS; ++j) cnt[j] += (s == uint32_t(j)) ? 1u : 0u;
+      }
     }
     // The tile's count of each digit: the two halves' counts added; the
     // first half's alone is where the second half's rows start.
 #pragma unroll
-    for (int j = 0; j < kMaxSplit; ++j) {
+    for (int j = 0; j < NS; ++j) {
       if (uint32_t(j) < S) {
         const uint32_t d = uint32_t(j) * L1 + (L - k);
         atomicAdd(&s_cnt[d], cnt[j]);
@@ -239,28 +244,40 @@ __global__ void __launch_bounds__(THREADS) k_list(const ListArgs a) {
   uint32_t* s_keys = s_stage;
   V* s_vals = reinterpret_cast<V*>(s_stage + stage_ids_at(a.stage_rows));
   if (act) {
-    uint32_t next[kMaxSplit];
+    uint32_t next[NS];
 #pragma unroll
-    for (int j = 0; j < kMaxSplit; ++j) {
+    for (int j = 0; j < NS; ++j) {
       const uint32_t d = uint32_t(j) * L1 + (L - k);
       next[j] = uint32_t(j) < S ? s_cnt[d] + (half ? s_half0[d] : 0u) : 0u;
     }
     const V kbits = V(k) << a.R.sym_bits;
-    auto place = [&](uint32_t i, uint32_t key, uint32_t prev) {
-      const uint32_t s = slice_of(a, key);
+    // (the terminator-only suffix, k = L, has no window but a base before it:
+    // its positions q are its reads' first, L before)
+    const bool has_prev = a.R.sym_bits && k != 0;
+    const uint32_t back = k < L ? 0u : L;
+    auto place = [&](uint32_t i) {
+      uint32_t prev = 0;
+      const uint32_t q = q0 + (i - ra) * L;
+      uint32_t key = window_staged(s_words, q, keep, has_prev && !back, &prev);
+      if (back && has_prev) {
+        const uint32_t qp = q + back - 1;
+        prev = (s_words[qp >> 4] >> (30u - 2u * (qp & 15u))) & 3u;
+      }
+      const uint32_t s = slice_of<NS>(a, key);
       if (s < S) {
         uint32_t r = 0;
 #pragma unroll
-        for (int j = 0; j < kMaxSplit; ++j)
+        for (int j = 0; j < NS; ++j)
           if (s == uint32_t(j)) r = next[j]++;
         s_keys[r] = key;
-        s_vals[r] = (V(i) << a.R.shift) | kbits | (a.R.sym_bits ? V(prev) : V(0));
+        s_vals[r] = (V(i) << a.R.shift) | kbits | V(prev);
       }
     };
-    for (uint32_t i = ra; i < rb; ++i) {
-      uint32_t prev;
-      const uint32_t key = window_staged(s_words, w_lo, uint64_t(i) * L, k, L, &prev);
-      place(i, key, prev);
+    if (NS == 1) {
+      for (; kept; kept &= kept - 1) place(ra + uint32_t(__ffsll((long long)kept)) - 1u);
+      for (uint32_t i = ra + 64u; i < rb; ++i) place(i);
+    } else {
+      for (uint32_t i = ra; i < rb; ++i) place(i);
     }
   }
   __syncthreads();
@@ -271,7 +288,7 @@ __global__ void __launch_bounds__(THREADS) k_list(const ListArgs a) {
   for (uint32_t r = uint32_t(tid); r < rows_kept; r += THREADS) {
     const uint32_t key = s_keys[r];
     const V v = s_vals[r];
-    const uint32_t s = slice_of(a, key);
+    const uint32_t s = slice_of<NS>(a, key);
     const uint32_t kk = (uint32_t(v) & kmask) >> a.R.sym_bits;
     const uint32_t d = s * L1 + (L - kk);
     const bool ok = s < S && kk <= L;
@@ -286,10 +303,10 @@ __global__ void __launch_bounds__(THREADS) k_list(const ListArgs a) {
   if (bad) atomicOr(a.err, kErrBounds);
 }
 
-template <class V, int THREADS>
+template <class V, int THREADS, int NS>
 cudaError_t launch_t(const ListArgs& a, cudaStream_t st) {
   const size_t smem = size_t(stage_ids_at(a.stage_rows)) * 4 + size_t(a.stage_rows) * sizeof(V);
-  auto kern = k_list<V, THREADS>;
+  auto kern = k_list<V, THREADS, NS>;
   static std::atomic<unsigned long long> configured{0};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -332,7 +349,8 @@ cudaError_t launch_list(const ListArgs& a, int id_bytes, cudaStream_t st) {
       a.stage_rows > kListMaxStage || a.stage_rows < a.reads_per_tile * L1 ||
       (uint64_t(a.reads_per_tile) * a.R.uniform_len + 15) / 16 + 2 > kListWords)
     return cudaErrorInvalidValue;
-  return id_bytes == 8 ? launch_t<uint64_t, 256>(a, st) : launch_t<uint32_t, 256>(a, st);
+  if (a.n_slices == 1) return id_bytes == 8 ? launch_t<uint64_t, 256, 1>(a, st) : launch_t<uint32_t, 256, 1>(a, st);
+  return id_bytes == 8 ? launch_t<uint64_t, 256, kMaxSplit>(a, st) : launch_t<uint32_t, 256, kMaxSplit>(a, st);
 }
 
 }  // namespace cxbwt
