@@ -760,6 +760,10 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     Slice sl;
     sl.rows = uint32_t(pl.N);
     slices.push_back(sl);
+    if (pl.groups && !depth) {
+      pl.depth = auto_depth(pl.N, pl.Lmax);
+      pl.seg_words = segsort_words(pl.Lmax, pl.depth);
+    }
   } else {
     if (!pl.groups)
       return fail(c, CXBWT_EUNSUPPORTED, "device-memory-bounded slices and parts use the group plan (reads of at most 528 bases)");

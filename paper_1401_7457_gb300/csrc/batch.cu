@@ -89,7 +89,7 @@ int build_pack(cxbwt_ctx* c, const cxbwt_collection* colls, const std::vector<ui
     if (!depth && tuned_choice(c, L, pl.N, &t_tile, &t_algo, &t_depth) && t_algo == CXBWT_ALGO_GROUPS)
       depth = t_depth;
   }
-  pl.depth = depth ? uint32_t(depth) : 16u;
+  pl.depth = depth ? uint32_t(depth) : auto_depth(pl.N, L);
   pl.seg_words = segsort_words(L, pl.depth);
   if (!pl.seg_words) {
     pl.depth = 16;

@@ -288,6 +288,17 @@ inline int take_device_error(cxbwt_ctx* c) {
 
 inline void* vptr(void* base, int idb, uint64_t row) { return static_cast<char*>(base) + row * uint64_t(idb); }
 
+// The group plan's depth l for N suffixes in one slice, where nothing asks for
+// another: each 4 bases less is a digit pass less, and pays while few suffixes
+// share their first l bases by chance (at most N / 4^l = 4 rows with 8 bases,
+// half a row with 12: 154k suffixes 141 us with l = 16, 119 with 8; 1.01M 170
+// and 160 with 12).
+inline uint32_t auto_depth(uint64_t n_suffixes, uint32_t max_len) {
+  const uint32_t d = n_suffixes <= (uint64_t(1) << 18) ? 8u : n_suffixes <= (uint64_t(1) << 23) ? 12u : 16u;
+  // (no wider keys for it than 16 words, whose group sorts hold fewer rows)
+  return max_len > d && segsort_words(max_len, d) && segsort_words(max_len, d) <= 16 ? d : 16u;
+}
+
 inline uint64_t tune_key(uint32_t max_len, uint64_t n_suffixes) {
   uint32_t cls = 0;
   while (cls < 63 && (uint64_t(1) << (cls + 1)) <= n_suffixes) ++cls;

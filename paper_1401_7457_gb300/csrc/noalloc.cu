@@ -27,10 +27,10 @@
 #include <mutex>
 
 #include "../../include/cxbwt.h"
-#include "group.cuh"
-#include "kernels.cuh"
+#include "host.cuh"
 
 using namespace cxbwt;
+using cxbwt::host::bits_for;
 
 namespace {
 
@@ -53,6 +53,7 @@ constexpr uint64_t kOffP = align256(kOffStatus + kMaxTiles * kRadix * 8);
 constexpr uint64_t kOffBase = align256(kOffP + uint64_t(kMaxLen) * kRadix * 4);
 // Reads of at most kMaxLen bases finish their groups with keys of at most
 // 16 words (segsort_words), which sets the CTA size of the group finish.
+// (auto_depth takes a depth below 16 only with such keys).
 static_assert((kMaxLen - 16 + 15) / 16 <= 16, "the group lists below assume keys of at most 16 words");
 constexpr uint64_t kCtaCap = cta_list_cap(kMaxRows), kBigCap = big_list_cap(kMaxRows, 16);
 // Look-back epochs one call may use: the four window-0 passes, then at most
@@ -79,11 +80,6 @@ uint32_t g_epoch[kMaxDevices] = {};    // look-back epoch, per device
     }                                   \
   } while (0)
 
-uint32_t bits_for(uint32_t x) {
-  uint32_t s = 0;
-  while (s < 32 && (uint64_t(1) << s) <= x) ++s;
-  return s;
-}
 
 }  // namespace
 
@@ -102,7 +98,8 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
   const uint64_t N = sum + n_reads;
   // Sizes beyond what the static array holds are rejected before any device work.
   if (N > kMaxRows || L > kMaxLen) return CXBWT_EUNSUPPORTED;
-  const int seg_words = segsort_words(L, 16);
+  const uint32_t depth = cxbwt::host::auto_depth(N, L);  // bases sorted by the digit passes
+  const int seg_words = segsort_words(L, depth);
   if (!seg_words) return CXBWT_EUNSUPPORTED;
 
   int dev = 0;
@@ -147,8 +144,8 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
   const uint64_t n_words = (sum + 15) / 16;
   ReadIndex R{reads_2bit, n_words, nullptr, shift, L, uint32_t(n_reads),
               (reinterpret_cast<uintptr_t>(reads_2bit) & 15u) == 0 ? 1u : 0u};
-  const uint32_t D = (L + 3) / 4, W = (L + 15) / 16;
-  const uint32_t d_sorted = std::min<uint32_t>(D, 4);
+  const uint32_t D = (L + 3) / 4;
+  const uint32_t d_sorted = std::min<uint32_t>(D, depth / 4);
   uint32_t* d_base = reinterpret_cast<uint32_t*>(base + kOffBase);
   int sm_count = 0;
   NA_CUDA(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
@@ -170,10 +167,10 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
   a.n_gen = N;
   a.n_out = uint32_t(N);
   a.n_tiles = uint32_t((N + kTile - 1) / kTile);
-  // Window 0 (bases 0..15): digit passes, least significant first; the first
+  // The first `depth` bases (of window 0): digit passes, least significant first; the first
   // generates the (length, read) start order.
   int cur = 0, kin = 0;
-  const uint32_t d_hi = std::min<uint32_t>(3, D - 1);
+  const uint32_t d_hi = d_sorted - 1;
   for (int64_t d = d_hi; d >= 0; --d) {
     const bool first = uint32_t(d) == d_hi;
     const int mode = first ? kSrcInitUniform : kSrcCarried;
@@ -190,14 +187,14 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
     cur ^= 1;
     kin = kout;
   }
-  if (L > 16) {
+  if (L > depth) {
     SegArgs g{};
     g.keys = keys[kin];
     g.vals = vals[cur];
     g.n_items = uint32_t(N);
     g.R = R;
-    g.depth = 16;
-    g.key_mask = depth_mask(16);
+    g.depth = depth;
+    g.key_mask = depth_mask(depth);
     g.cta_list = reinterpret_cast<uint2*>(base + kOffSeg);
     g.cta_cap = uint32_t(kCtaCap);
     g.big_list = g.cta_list + kCtaCap;
@@ -214,9 +211,9 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
       uint2 bg;
       NA_CUDA(cudaMemcpyAsync(&bg, g.big_list + b, 8, cudaMemcpyDeviceToHost, st));
       NA_CUDA(cudaStreamSynchronize(st));
-      const uint32_t s0 = bg.x, m = bg.y, n_win = W - 1;
+      const uint32_t s0 = bg.x, m = bg.y, n_win = (L - depth + 15) / 16;
       NA_CUDA(cudaMemsetAsync(rh, 0, size_t(n_win) * 4 * kRadix * 4, st));
-      NA_CUDA(launch_range_hist(static_cast<uint32_t*>(vals[cur]) + s0, 4, m, R, 16, n_win, rh, sm_count, st));
+      NA_CUDA(launch_range_hist(static_cast<uint32_t*>(vals[cur]) + s0, 4, m, R, depth, n_win, rh, sm_count, st));
       void* gv[2] = {static_cast<uint32_t*>(vals[cur]) + s0, static_cast<uint32_t*>(vals[cur ^ 1]) + s0};
       uint32_t* gk[2] = {keys[0] + s0, keys[1] + s0};
       int gc = 0, gki = 0;
@@ -224,19 +221,19 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
       b2.n_gen = m;
       b2.n_out = m;
       b2.n_tiles = (m + kTile - 1) / kTile;
-      for (uint32_t w = W - 1; w >= 1; --w) {
-        const uint32_t lo = 4 * w, hi = std::min<uint32_t>(lo + 3, D - 1);
-        for (int64_t d = hi; d >= int64_t(lo); --d) {
-          const bool first_in = uint32_t(d) == hi, last_in = uint32_t(d) == lo;
+      for (uint32_t u = n_win; u-- > 0;) {  // windows of bases depth + 16 u ..
+        const uint32_t c0 = depth + 16 * u, n_dig = std::min<uint32_t>(4, (L - c0 + 3) / 4);
+        for (uint32_t j = n_dig; j-- > 0;) {
+          const bool first_in = j == n_dig - 1, last_in = j == 0;
           const int mode = first_in ? kSrcExtract : kSrcCarried;
           b2.vals_in = gv[gc];
           b2.vals_out = gv[gc ^ 1];
           b2.keys_in = mode == kSrcCarried ? gk[gki] : nullptr;
           const int kout = mode == kSrcCarried ? (gki ^ 1) : gki;
           b2.keys_out = last_in ? nullptr : gk[kout];
-          b2.digit_base = rh + size_t((w - 1) * 4 + (uint32_t(d) - lo)) * kRadix;
-          b2.key_shift = 24u - 8u * (uint32_t(d) - lo);
-          b2.window_c0 = 16 * w;
+          b2.digit_base = rh + size_t(u * 4 + j) * kRadix;
+          b2.key_shift = 24u - 8u * j;
+          b2.window_c0 = c0;
           b2.epoch = ++epoch;
           NA_CUDA(launch_onesweep(b2, mode, !last_in, false, 4, shape, st));
           gc ^= 1;
