@@ -661,7 +661,7 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   pl.w_last = pl.groups ? 0u : pl.W - 1;
   plan_ids(pl, (c->opt.plan_flags & CXBWT_PLAN_ID64) != 0,
            pl.n_words * 4 > (64u << 20) || (c->opt.plan_flags & CXBWT_PLAN_CARRY_BASE));
-  r.shape = onesweep_shape(tile_items, pl.idb);
+  r.shape = onesweep_shape(!tile_items && pl.N <= kSmallRows ? kSmallTile : tile_items, pl.idb);
   const uint32_t TILE = uint32_t(r.shape.tile());
 
   // ---- inputs on the device ----------------------------------------------

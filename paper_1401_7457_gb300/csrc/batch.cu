@@ -98,7 +98,7 @@ int build_pack(cxbwt_ctx* c, const cxbwt_collection* colls, const std::vector<ui
   pl.groups = true;
   pl.w_last = 0;
   plan_ids(pl, (c->opt.plan_flags & CXBWT_PLAN_ID64) != 0, (c->opt.plan_flags & CXBWT_PLAN_CARRY_BASE) != 0);
-  r.shape = onesweep_shape(c->opt.tile_items, pl.idb);
+  r.shape = onesweep_shape(!c->opt.tile_items && pl.N <= kSmallRows ? kSmallTile : c->opt.tile_items, pl.idb);
   const uint32_t TILE = uint32_t(r.shape.tile());
 
   // ---- pack store, descriptors ---------------------------------------------

@@ -5,6 +5,8 @@
 namespace cxbwt {
 
 TileShape onesweep_shape(int tile_items_hint, int id_bytes) {
+  if (id_bytes == 4 && tile_items_hint == kSmallTile)
+    return TileShape{onesweep::ShapeSmall::threads, onesweep::ShapeSmall::ipt};
   if (id_bytes == 4 && tile_items_hint == 8192)
     return TileShape{onesweep::ShapeLarge::threads, onesweep::ShapeLarge::ipt};
   if (id_bytes == 8 && tile_items_hint == 2048)
@@ -22,6 +24,7 @@ cudaError_t launch_onesweep_t<uint32_t>(const PassArgs& a, int mode, bool wk, bo
   if (a.n_tiles == 0) return cudaSuccess;
   if (s.threads == onesweep::ShapeLarge::threads && s.items_per_thread == onesweep::ShapeLarge::ipt)
     return onesweep::launch_shape<uint32_t, onesweep::ShapeLarge>(a, mode, wk, filter, st);
+  if (s.items_per_thread == onesweep::ShapeSmall::ipt) return launch_onesweep32_small(a, mode, wk, filter, st);
   return onesweep::launch_shape<uint32_t, onesweep::ShapeMid>(a, mode, wk, filter, st);
 }
 

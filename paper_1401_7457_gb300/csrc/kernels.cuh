@@ -113,6 +113,10 @@ struct TileShape {
   int tile() const { return threads * items_per_thread; }
 };
 TileShape onesweep_shape(int tile_items_hint, int id_bytes);
+// Tiles of collections of at most kSmallRows suffixes (32-bit ids).
+constexpr int kSmallTile = 1024;
+constexpr uint64_t kSmallRows = uint64_t(1) << 19;
+cudaError_t launch_onesweep32_small(const PassArgs& a, int mode, bool wk, bool filter, cudaStream_t st);
 // id_bytes: 4 or 8.  filter: drop rows outside the bucket range (generated modes only).
 cudaError_t launch_onesweep(const PassArgs& a, int mode, bool write_key, bool filter, int id_bytes,
                             const TileShape& shape, cudaStream_t st);

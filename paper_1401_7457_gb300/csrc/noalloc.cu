@@ -36,8 +36,9 @@ namespace {
 
 constexpr uint64_t kMaxRows = CXBWT_NOALLOC_MAX_SUFFIXES;
 constexpr uint32_t kMaxLen = CXBWT_NOALLOC_MAX_READ_LEN;
-constexpr uint32_t kTile = 4096;                       // onesweep_shape(0, 4).tile(), checked at each call
-constexpr uint64_t kMaxTiles = (kMaxRows + kTile - 1) / kTile;
+// Tiles of up to kSmallRows rows, and above (checked at each call).
+constexpr uint32_t kTileSmall = kSmallTile, kTileLarge = 4096;
+constexpr uint64_t kMaxTiles = std::max((kMaxRows + kTileLarge - 1) / kTileLarge, (kSmallRows + kTileSmall - 1) / kTileSmall);
 constexpr uint32_t kMaxD = (kMaxLen + 3) / 4;
 constexpr uint32_t kMaxW = (kMaxLen + 15) / 16;
 
@@ -155,8 +156,9 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
 
   void* vals[2] = {base + kOffVals0, base + kOffVals1};
   uint32_t* keys[2] = {reinterpret_cast<uint32_t*>(base + kOffKeys0), reinterpret_cast<uint32_t*>(base + kOffKeys1)};
-  const TileShape shape = onesweep_shape(0, 4);
-  if (uint32_t(shape.tile()) != kTile) return CXBWT_EINTERNAL;  // the array was sized for kTile-item tiles
+  const TileShape shape = onesweep_shape(N <= kSmallRows ? kSmallTile : 0, 4);
+  const uint32_t kTile = N <= kSmallRows ? kTileSmall : kTileLarge;
+  if (uint32_t(shape.tile()) != kTile) return CXBWT_EINTERNAL;  // the array was sized for these tiles
   PassArgs a{};
   a.status = reinterpret_cast<unsigned long long*>(base + kOffStatus);
   a.tile_counter = d_counter;

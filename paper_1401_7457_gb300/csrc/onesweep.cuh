@@ -478,6 +478,7 @@ struct Shape {
   static constexpr int threads = T, ipt = I, min_blocks = B;
 };
 using ShapeMid = Shape<256, 16, 4>;    // 4096 items
+using ShapeSmall = Shape<256, 4, 6>;   // 1024 items (32-bit ids, small collections)
 using ShapeLarge = Shape<512, 16, 2>;  // 8192 items (32-bit ids)
 using Shape64x16 = Shape<256, 16, 3>;  // 4096 items, 64-bit ids: 48 KB staged holds an SM to three CTAs,
                                        // so the registers are sized for three (no spills)
