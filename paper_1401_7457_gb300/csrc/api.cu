@@ -56,6 +56,71 @@ static uint64_t status_tiles(const cxbwt_ctx* c, const Plan& pl, uint32_t TILE) 
   return t;
 }
 
+// Finishes the groups of r.big_g that were too large for one CTA, whose number
+// the completed copy of the group counts in h_small gives, with LSD passes over
+// bases l.. restricted to their rows.  *any: there were some.
+static int finish_big_groups(cxbwt_ctx* c, Run& r, bool* any) {
+  const Plan& pl = r.pl;
+  cudaStream_t st = r.st;
+  const SegArgs& g = r.big_g;
+  const PassArgs& a = r.big_a;
+  const int idb = pl.idb, cur = r.big_cur;
+  const uint32_t TILE = uint32_t(r.shape.tile());
+  const uint32_t n_big = std::min<uint32_t>(reinterpret_cast<const uint32_t*>(c->h_small + 5)[1], g.big_cap);
+  c->stats.cta_groups += uint64_t(reinterpret_cast<const uint32_t*>(c->h_small + 5)[0]) +
+                         reinterpret_cast<const uint32_t*>(c->h_small + 5)[3];
+  c->stats.big_groups += n_big;
+  if (n_big) {
+    std::vector<uint2> big(n_big);
+    CX_CUDA(c, cudaMemcpyAsync(big.data(), g.big_list, n_big * 8, cudaMemcpyDeviceToHost, st));
+    CX_CUDA(c, cudaStreamSynchronize(st));
+    r.d2h += n_big * 8;
+    // Windows of bases [l + 16u, l + 16u + 16), u < n_win, cover bases l .. Lmax-1.
+    const uint32_t n_win = (pl.Lmax - pl.depth + 15) / 16;
+    auto* rh = static_cast<uint32_t*>(c->rhist.p);
+    for (const uint2& bg : big) {
+      const uint32_t s0 = bg.x, m = bg.y;
+      CX_CUDA(c, cudaMemsetAsync(rh, 0, size_t(n_win) * 4 * kRadix * 4, st));
+      CX_CUDA(c, launch_range_hist(vptr(r.vals[cur], idb, s0), idb, m, r.R, pl.depth, n_win, rh, c->sm_count, st));
+      r.launches += 2;
+      void* gv[2] = {vptr(r.vals[cur], idb, s0), vptr(r.vals[cur ^ 1], idb, s0)};
+      uint32_t* gk[2] = {r.keys[0] + s0, r.keys[1] + s0};
+      int gc = 0, gki = 0;
+      PassArgs b = a;
+      b.n_gen = m;
+      b.n_out = m;
+      b.n_tiles = uint32_t((m + TILE - 1) / TILE);
+      for (uint32_t u = n_win; u-- > 0;) {
+        const uint32_t c0 = pl.depth + 16 * u;
+        const uint32_t n_dig = std::min<uint32_t>(4, (pl.Lmax - c0 + 3) / 4);  // digits holding bases < Lmax
+        for (int64_t j = int64_t(n_dig) - 1; j >= 0; --j) {
+          const bool first_in_window = (uint32_t(j) == n_dig - 1);
+          const bool last_in_window = (j == 0);
+          const int mode = first_in_window ? kSrcExtract : kSrcCarried;
+          const bool write_key = !last_in_window;
+          b.vals_in = gv[gc];
+          b.vals_out = gv[gc ^ 1];
+          b.keys_in = (mode == kSrcCarried) ? gk[gki] : nullptr;
+          const int kout = (mode == kSrcCarried) ? (gki ^ 1) : gki;
+          b.keys_out = write_key ? gk[kout] : nullptr;
+          b.digit_base = rh + size_t(u * 4 + uint32_t(j)) * kRadix;
+          b.key_shift = 24u - 8u * uint32_t(j);
+          b.window_c0 = c0;
+          b.epoch = ++c->epoch;
+          CX_CUDA(c, launch_onesweep(b, mode, write_key, false, idb, r.shape, st));
+          gc ^= 1;
+          if (write_key) gki = kout;
+          ++r.sort_launches;
+          r.sort_items += m;
+        }
+      }
+      if (gc) CX_CUDA(c, cudaMemcpyAsync(gv[0], gv[1], size_t(m) * idb, cudaMemcpyDeviceToDevice, st));
+    }
+  }
+  *any = n_big != 0;
+  return CXBWT_OK;
+}
+
 // Sort the slice's suffixes into r.vals[cur]; returns cur (0 or 1) through
 // *cur_out.  tev (or nullptr): events recorded before the digit passes and
 // after them.
@@ -302,59 +367,19 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
     CX_CUDA(c, launch_segsort(g, pl.seg_words, idb, c->sm_count, pl.n_words * 4 > (64u << 20), st));
     r.launches += 2;
     // Remainders too large for one CTA (rare: long runs of equal bases) are
-    // finished here with LSD passes over bases l.. restricted to their rows.
+    // finished by the host's launches, once it has read how many there are:
+    // now, or (r.defer) when it reads the end of the build, which then writes
+    // the outputs a second time if there are any (1.01M suffixes: a round trip
+    // less, 5 us of 160).
     CX_CUDA(c, cudaMemcpyAsync(c->h_small + 5, r.d_seg, 16, cudaMemcpyDeviceToHost, st));
-    CX_CUDA(c, cudaStreamSynchronize(st));
-    const uint32_t n_big = std::min<uint32_t>(reinterpret_cast<const uint32_t*>(c->h_small + 5)[1], g.big_cap);
-    c->stats.cta_groups += uint64_t(reinterpret_cast<const uint32_t*>(c->h_small + 5)[0]) +
-                           reinterpret_cast<const uint32_t*>(c->h_small + 5)[3];
-    c->stats.big_groups += n_big;
-    if (n_big) {
-      std::vector<uint2> big(n_big);
-      CX_CUDA(c, cudaMemcpyAsync(big.data(), g.big_list, n_big * 8, cudaMemcpyDeviceToHost, st));
+    r.big_g = g;
+    r.big_a = a;
+    r.big_cur = cur;
+    r.deferred = r.defer;
+    if (!r.defer) {
       CX_CUDA(c, cudaStreamSynchronize(st));
-      r.d2h += n_big * 8;
-      // Windows of bases [l + 16u, l + 16u + 16), u < n_win, cover bases l .. Lmax-1.
-      const uint32_t n_win = (pl.Lmax - pl.depth + 15) / 16;
-      auto* rh = static_cast<uint32_t*>(c->rhist.p);
-      for (const uint2& bg : big) {
-        const uint32_t s0 = bg.x, m = bg.y;
-        CX_CUDA(c, cudaMemsetAsync(rh, 0, size_t(n_win) * 4 * kRadix * 4, st));
-        CX_CUDA(c, launch_range_hist(vptr(r.vals[cur], idb, s0), idb, m, r.R, pl.depth, n_win, rh, c->sm_count, st));
-        r.launches += 2;
-        void* gv[2] = {vptr(r.vals[cur], idb, s0), vptr(r.vals[cur ^ 1], idb, s0)};
-        uint32_t* gk[2] = {r.keys[0] + s0, r.keys[1] + s0};
-        int gc = 0, gki = 0;
-        PassArgs b = a;
-        b.n_gen = m;
-        b.n_out = m;
-        b.n_tiles = uint32_t((m + TILE - 1) / TILE);
-        for (uint32_t u = n_win; u-- > 0;) {
-          const uint32_t c0 = pl.depth + 16 * u;
-          const uint32_t n_dig = std::min<uint32_t>(4, (pl.Lmax - c0 + 3) / 4);  // digits holding bases < Lmax
-          for (int64_t j = int64_t(n_dig) - 1; j >= 0; --j) {
-            const bool first_in_window = (uint32_t(j) == n_dig - 1);
-            const bool last_in_window = (j == 0);
-            const int mode = first_in_window ? kSrcExtract : kSrcCarried;
-            const bool write_key = !last_in_window;
-            b.vals_in = gv[gc];
-            b.vals_out = gv[gc ^ 1];
-            b.keys_in = (mode == kSrcCarried) ? gk[gki] : nullptr;
-            const int kout = (mode == kSrcCarried) ? (gki ^ 1) : gki;
-            b.keys_out = write_key ? gk[kout] : nullptr;
-            b.digit_base = rh + size_t(u * 4 + uint32_t(j)) * kRadix;
-            b.key_shift = 24u - 8u * uint32_t(j);
-            b.window_c0 = c0;
-            b.epoch = ++c->epoch;
-            CX_CUDA(c, launch_onesweep(b, mode, write_key, false, idb, r.shape, st));
-            gc ^= 1;
-            if (write_key) gki = kout;
-            ++r.sort_launches;
-            r.sort_items += m;
-          }
-        }
-        if (gc) CX_CUDA(c, cudaMemcpyAsync(gv[0], gv[1], size_t(m) * idb, cudaMemcpyDeviceToDevice, st));
-      }
+      bool any = false;
+      CX_TRY(finish_big_groups(c, r, &any));
     }
   }
   *cur_out = cur;
@@ -467,21 +492,42 @@ static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_
   const Plan& pl = r.pl;
   cudaStream_t st = r.st;
   const bool timing = c->opt.timing != 0;
-  if (timing) CX_CUDA(c, cudaEventRecord(c->ev[3], st));
-  if (!o.bwt_dev) {
-    CX_CUDA(c, cudaEventRecord(c->slice_done[0], c->side));
-    CX_CUDA(c, cudaStreamWaitEvent(st, c->slice_done[0], 0));
+  const bool host_out = !o.bwt_dev || (o.dollar && !o.dollar_dev) || (o.counts && !o.counts_dev) || (o.sa && !o.sa_dev);
+  const bool wait = !c->opt.async || host_out;
+  for (;;) {
+    if (timing) CX_CUDA(c, cudaEventRecord(c->ev[3], st));
+    if (!o.bwt_dev) {
+      CX_CUDA(c, cudaEventRecord(c->slice_done[0], c->side));
+      CX_CUDA(c, cudaStreamWaitEvent(st, c->slice_done[0], 0));
+    }
+    if (o.counts) {
+      CX_CUDA(c, cudaMemcpyAsync(o.counts, r.d_counts, 5 * 8, o.counts_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
+                                 st));
+      if (!o.counts_dev) r.d2h += 40;
+    }
+    if (o.dollar && !o.dollar_dev) {
+      CX_CUDA(c, cudaMemcpyAsync(o.dollar, r.d_dollar, pl.n * 8, cudaMemcpyDeviceToHost, st));
+      r.d2h += pl.n * 8;
+    }
+    CX_CUDA(c, cudaMemcpyAsync(c->h_small + 4, r.d_err, 4, cudaMemcpyDeviceToHost, st));
+    if (!wait) break;
+    CX_CUDA(c, cudaStreamSynchronize(st));
+    CX_TRY(take_device_error(c));
+    if (!r.deferred) break;
+    // The group counts have come with the rest.
+    r.deferred = false;
+    bool any = false;
+    CX_TRY(finish_big_groups(c, r, &any));
+    if (!any) break;
+    CX_CUDA(c, cudaMemsetAsync(r.d_counts, 0, 5 * 8, st));
+    CX_CUDA(c, launch_emit(r.emitted, st));
+    r.launches += r.emitted.sa_out ? 2 : 1;
+    if (!o.bwt_dev) {
+      const uint64_t words = (pl.N + 15) / 16;
+      CX_CUDA(c, cudaMemcpyAsync(o.bwt, r.d_bwt, words * 4, cudaMemcpyDeviceToHost, st));
+      r.d2h += words * 4;
+    }
   }
-  if (o.counts) {
-    CX_CUDA(c, cudaMemcpyAsync(o.counts, r.d_counts, 5 * 8, o.counts_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                               st));
-    if (!o.counts_dev) r.d2h += 40;
-  }
-  if (o.dollar && !o.dollar_dev) {
-    CX_CUDA(c, cudaMemcpyAsync(o.dollar, r.d_dollar, pl.n * 8, cudaMemcpyDeviceToHost, st));
-    r.d2h += pl.n * 8;
-  }
-  CX_CUDA(c, cudaMemcpyAsync(c->h_small + 4, r.d_err, 4, cudaMemcpyDeviceToHost, st));
 
   c->stats.kernel_launches += r.launches + r.sort_launches;
   c->stats.sort_pass_launches += r.sort_launches;
@@ -494,16 +540,13 @@ static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_
   c->stats.carried_pass_items += r.carried_items;
   c->stats.merge_launches += r.merge_launches;
 
-  const bool host_out = !o.bwt_dev || (o.dollar && !o.dollar_dev) || (o.counts && !o.counts_dev) || (o.sa && !o.sa_dev);
-  if (c->opt.async && !host_out) {
+  if (!wait) {
     // Completed (and checked) by cxbwt_sync.
     c->stats.builds += 1;
     c->stats.bases += pl.sum;
     c->stats.suffixes += pl.N;
     return CXBWT_OK;
   }
-  CX_CUDA(c, cudaStreamSynchronize(st));
-  CX_TRY(take_device_error(c));
   if (timing) {
     float ms_all = 0;
     CX_CUDA(c, cudaEventElapsedTime(&ms_all, c->ev[0], c->ev[3]));
@@ -1037,6 +1080,9 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
       r.vals[0] = vptr(c->vals[0].p, pl.idb, sl.arr0);
       r.keys[0] = static_cast<uint32_t*>(c->keys[0].p) + sl.arr0;
     }
+    // (slices' edge words are merged into their neighbours', and a host suffix
+    // list is copied slice by slice: neither is written twice)
+    r.defer = slices.size() == 1 && sl.whole && !c->opt.async && !(out_sa && !sa_dev);
     CX_TRY(sort_slice(c, r, sl, &cur, tev));
     if (tev) CX_CUDA(c, cudaEventRecord(tev[2], st));
     // ---- emission of the slice -------------------------------------------
@@ -1056,6 +1102,7 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     e.read_base = 0;
     e.n_reads_out = uint32_t(n);
     CX_CUDA(c, launch_emit(e, st));
+    r.emitted = e;
     r.launches += e.sa_out ? 2 : 1;
     if (tev) CX_CUDA(c, cudaEventRecord(tev[3], st));
     if (out_sa && !sa_dev) {

@@ -247,6 +247,13 @@ struct Run {
   uint64_t launches = 0, sort_launches = 0, sort_items = 0, d2h = 0;
   uint64_t carried_launches = 0, carried_items = 0;
   uint64_t merge_launches = 0;
+  // The groups too large for one CTA: what their finish needs, and whether it
+  // is left to the end of the build (which then emits again: emitted).
+  bool defer = false, deferred = false;
+  SegArgs big_g{};
+  PassArgs big_a{};
+  int big_cur = 0;
+  EmitArgs emitted{};
   // Per-pass timing (timing option): pass j ran between events pev[2j] and
   // pev[2j+1]; pev_carried[j] says whether it was a carried-key pass.
   uint32_t n_pev = 0;
