@@ -144,11 +144,12 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
   // whole: rows 0..d_sorted-1 = char digits d, rows D.. = length digits.
   // slice: row 0 = suffix length (its low byte), rows 1..4 = window-0 digits
   // (most significant first), row 5 = the high byte of the suffix length.
-  // A slice of whole 4-base buckets listed by the listing kernel: its digits
-  // are counted from the listed keys (4 bytes each) instead of by a scan of
-  // every suffix of the collection (505M suffixes in three slices: 1.52 ms a
-  // slice, against 0.25 ms for its 168M keys).
-  const bool count_listed = r.P_host && !sl.whole && !sl.pregen && pl.uniform && r.read_major && list_kernel(c, pl);
+  // A slice listed by the listing kernel: its digits are counted from the
+  // listed keys (4 bytes each) instead of by a scan of every suffix of the
+  // collection (505M suffixes in three slices: 1.52 ms a slice, against 0.25 ms
+  // for its 168M keys), its suffix lengths from the counts that planned whole
+  // 4-base buckets, or by a walk over the store that counts nothing else.
+  const bool count_listed = !sl.whole && !sl.pregen && pl.uniform && r.read_major && list_kernel(c, pl);
   if (sl.pregen) {
     // The slice's first windows are listed already: count their digits (rows 1..4).
     CX_CUDA(c, cudaMemsetAsync(r.base + kRadix, 0, 4 * kRadix * 4, st));
@@ -160,7 +161,7 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
     CX_CUDA(c, launch_digitbase(static_cast<const uint32_t*>(c->P.p), pl.Lmax, d_sorted, pl.uniform ? 1 : 0,
                                 uint32_t(pl.n), pl.Lmax, static_cast<const uint32_t*>(c->lenhist.p), r.base, st));
     r.launches += 2;
-  } else if (count_listed) {
+  } else if (count_listed && r.P_host) {
     // Suffixes per length of the slice's 4-base buckets: of length t, those
     // whose 4-mer at position L - t is in the slice; the terminator-only ones
     // are in bucket 0.  The window digits are counted once the slice is listed.
@@ -174,6 +175,11 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
     if (acc != sl.rows)
       return fail(c, CXBWT_EINTERNAL, "a slice of %u suffixes, %llu by length", sl.rows, (unsigned long long)acc);
     CX_CUDA(c, cudaMemcpyAsync(r.base, first.data(), kRadix * 4, cudaMemcpyHostToDevice, st));
+  } else if (count_listed) {
+    CX_CUDA(c, cudaMemsetAsync(r.base, 0, kRadix * 4, st));
+    CX_CUDA(c, launch_list_lengths(r.R, uint32_t(pl.n), sl.key_lo, a.key_last, r.base, c->sm_count, st));
+    CX_CUDA(c, launch_scan_rows(r.base, 1, st));
+    r.launches += 2;
   } else {
     CX_CUDA(c, cudaMemsetAsync(r.base, 0, 6 * kRadix * 4, st));
     CX_CUDA(c, launch_pass_hist(r.R, uint32_t(pl.n), sl.key_lo, uint32_t(sl.key_hi - 1 - sl.key_lo), r.base,

@@ -331,6 +331,11 @@ cudaError_t launch_sub_bucket_hist(const ReadIndex& R, uint32_t n_reads, uint32_
   return cudaGetLastError();
 }
 
+cudaError_t launch_scan_rows(uint32_t* hist, uint32_t rows, cudaStream_t st) {
+  k_scan_rows<<<rows, kRadix, 0, st>>>(hist);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_pass_hist(const ReadIndex& R, uint32_t n_reads, uint32_t key_lo, uint32_t key_last,
                              uint32_t* hist, int sm_count, cudaStream_t st) {
   uint32_t gx = (n_reads + 511) / 512;

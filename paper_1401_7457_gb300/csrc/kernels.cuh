@@ -105,6 +105,12 @@ struct ListArgs {
 };
 uint32_t list_reads_per_tile(uint32_t read_len);
 cudaError_t launch_list(const ListArgs& a, int id_bytes, cudaStream_t st);
+// Suffixes of each length, of reads of one length (at most 255) whose first
+// window w has w - key_lo <= key_last: added to hist[0 .. L].
+cudaError_t launch_list_lengths(const ReadIndex& R, uint32_t n_reads, uint32_t key_lo, uint32_t key_last, uint32_t* hist,
+                                int sm_count, cudaStream_t st);
+// hist[256 * r ..] becomes its exclusive prefix sums, for r < rows.
+cudaError_t launch_scan_rows(uint32_t* hist, uint32_t rows, cudaStream_t st);
 
 // Tile geometry of the digit pass (threads x items per thread).
 struct TileShape {
