@@ -140,6 +140,8 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
   a.prefetch = (c->opt.plan_flags & CXBWT_PLAN_NO_PREFETCH) ? 0u : 1u;
   const uint32_t d_sorted = std::min<uint32_t>(pl.D, 4 * (pl.w_last + 1));
 
+  if (pl.groups && pl.Lmax > pl.depth) CX_CUDA(c, cudaMemsetAsync(r.d_seg, 0, 32, st));  // the group finish's counters
+
   // ---- digit bases -----------------------------------------------------------
   // whole: rows 0..d_sorted-1 = char digits d, rows D.. = length digits.
   // slice: row 0 = suffix length (its low byte), rows 1..4 = window-0 digits
@@ -356,7 +358,6 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
   // ---- group plan: finish every group of equal first l bases on chip --------
   if (pl.groups && pl.Lmax > pl.depth) {
     const uint64_t cta_cap = cta_list_cap(sl.rows), big_cap = big_list_cap(sl.rows, pl.seg_words);
-    CX_CUDA(c, cudaMemsetAsync(r.d_seg, 0, 32, st));
     SegArgs g{};
     g.keys = r.keys[kin];
     g.vals = r.vals[cur];
@@ -377,12 +378,12 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
     // now, or (r.defer) when it reads the end of the build, which then writes
     // the outputs a second time if there are any (1.01M suffixes: a round trip
     // less, 5 us of 160).
-    CX_CUDA(c, cudaMemcpyAsync(c->h_small + 5, r.d_seg, 16, cudaMemcpyDeviceToHost, st));
     r.big_g = g;
     r.big_a = a;
     r.big_cur = cur;
     r.deferred = r.defer;
     if (!r.defer) {
+      CX_CUDA(c, cudaMemcpyAsync(c->h_small + 5, r.d_seg, 16, cudaMemcpyDeviceToHost, st));
       CX_CUDA(c, cudaStreamSynchronize(st));
       bool any = false;
       CX_TRY(finish_big_groups(c, r, &any));
@@ -516,6 +517,7 @@ static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_
       r.d2h += pl.n * 8;
     }
     CX_CUDA(c, cudaMemcpyAsync(c->h_small + 4, r.d_err, 4, cudaMemcpyDeviceToHost, st));
+    if (r.deferred) CX_CUDA(c, cudaMemcpyAsync(c->h_small + 5, r.d_seg, 16, cudaMemcpyDeviceToHost, st));
     if (!wait) break;
     CX_CUDA(c, cudaStreamSynchronize(st));
     CX_TRY(take_device_error(c));

@@ -23,6 +23,8 @@ template <class V>
 __global__ void __launch_bounds__(kEmitThreads) k_emit(const EmitArgs a) {
   __shared__ unsigned long long s_cnt[5];
   if (threadIdx.x < 5) s_cnt[threadIdx.x] = 0;
+  grid_dependency_wait();
+  grid_launch_dependents();
   __syncthreads();
   const V* sa = static_cast<const V*>(a.sa);
   const uint64_t w = (a.row0 >> 4) + uint64_t(blockIdx.x) * blockDim.x + threadIdx.x;  // global word
@@ -44,7 +46,7 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(const EmitArgs a) {
       const uint4* p = reinterpret_cast<const uint4*>(sa + (g0 - a.row0));
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const uint4 x = __ldg(p + q);
+        const uint4 x = p[q];
         v[4 * q] = V(x.x); v[4 * q + 1] = V(x.y); v[4 * q + 2] = V(x.z); v[4 * q + 3] = V(x.w);
       }
     } else if (full16 && aligned16 && sizeof(V) == 8) {
@@ -52,7 +54,7 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(const EmitArgs a) {
       const uint4* p = reinterpret_cast<const uint4*>(sa + (g0 - a.row0));
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
-        const uint4 x = __ldg(p + q);
+        const uint4 x = p[q];
         v[2 * q] = V((uint64_t(x.y) << 32) | x.x);
         v[2 * q + 1] = V((uint64_t(x.w) << 32) | x.z);
       }
@@ -104,11 +106,13 @@ __global__ void __launch_bounds__(kEmitThreads) k_emit(const EmitArgs a) {
 template <class V>
 __global__ void __launch_bounds__(kEmitThreads) k_emit_sa(const EmitArgs a) {
   constexpr int kRows = 4;
+  grid_dependency_wait();
+  grid_launch_dependents();
   const V* sa = static_cast<const V*>(a.sa);
   const uint64_t r0 = uint64_t(blockIdx.x) * (kEmitThreads * kRows) + threadIdx.x;
   V v[kRows];
 #pragma unroll
-  for (int j = 0; j < kRows; ++j) v[j] = r0 + j * kEmitThreads < a.n ? __ldg(sa + r0 + j * kEmitThreads) : V(0);
+  for (int j = 0; j < kRows; ++j) v[j] = r0 + j * kEmitThreads < a.n ? sa[r0 + j * kEmitThreads] : V(0);
 #pragma unroll
   for (int j = 0; j < kRows; ++j) {
     const uint64_t r = r0 + j * kEmitThreads;
@@ -126,14 +130,11 @@ cudaError_t launch_emit(const EmitArgs& a, cudaStream_t st) {
   const uint64_t blocks = (words + kEmitThreads - 1) / kEmitThreads;
   if (a.sa_out) {
     const uint64_t sa_blocks = (uint64_t(a.n) + kEmitThreads * 4 - 1) / (kEmitThreads * 4);
-    if (a.id_bytes == 8) k_emit_sa<uint64_t><<<uint32_t(sa_blocks), kEmitThreads, 0, st>>>(a);
-    else k_emit_sa<uint32_t><<<uint32_t(sa_blocks), kEmitThreads, 0, st>>>(a);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_after(a.n < kEarlyRows, a.id_bytes == 8 ? k_emit_sa<uint64_t> : k_emit_sa<uint32_t>, dim3(uint32_t(sa_blocks)),
+                                       kEmitThreads, 0, st, a);
     if (e != cudaSuccess) return e;
   }
-  if (a.id_bytes == 8) k_emit<uint64_t><<<uint32_t(blocks), kEmitThreads, 0, st>>>(a);
-  else k_emit<uint32_t><<<uint32_t(blocks), kEmitThreads, 0, st>>>(a);
-  return cudaGetLastError();
+  return launch_after(a.n < kEarlyRows, a.id_bytes == 8 ? k_emit<uint64_t> : k_emit<uint32_t>, dim3(uint32_t(blocks)), kEmitThreads, 0, st, a);
 }
 
 }  // namespace cxbwt

@@ -322,6 +322,8 @@ __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
   using H = typename Heads<SPAN>::T;
   const int lane = threadIdx.x & 31;
   __shared__ RowWords<NW, SPAN> s_rows[8];
+  grid_dependency_wait();
+  grid_launch_dependents();
   RowWords<NW, SPAN>& sw = s_rows[threadIdx.x >> 5];
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t chunk = a.chunk, n_chunks = (a.n_items + chunk - 1) / chunk;
@@ -390,6 +392,8 @@ __global__ void __launch_bounds__(THREADS) k_segsort_cta(const SegArgs a, const 
   uint32_t* s_w = reinterpret_cast<uint32_t*>(s_v + kRows);         // [NW][kRows]
   uint16_t* s_perm = reinterpret_cast<uint16_t*>(s_w + NW * kRows);  // [kRows]
   __shared__ uint32_t s_item;
+  grid_dependency_wait();
+  grid_launch_dependents();
   const uint32_t n_list = min(*(volatile const uint32_t*)n_ptr, cap);
   for (;;) {
     __syncthreads();
@@ -505,7 +509,7 @@ cudaError_t launch_cta_nw(const SegArgs& a, uint32_t grid, const uint2* list, co
     if (e != cudaSuccess) return e;
     configured.fetch_or(bit, std::memory_order_release);
   }
-  kern<<<grid, THREADS, smem, st>>>(a, list, n_ptr, cap, dir, work);
+  return launch_after(a.n_items < kEarlyRows, kern, dim3(grid), THREADS, smem, st, a, list, n_ptr, cap, dir, work);
   return cudaGetLastError();
 }
 
@@ -521,9 +525,7 @@ cudaError_t launch_nw(const SegArgs& args, int sm_count, bool wide, cudaStream_t
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
   // Rows of the widest keys (long reads) would not fit twice in shared memory.
-  if (wide && NW <= 16) k_segsort_warp_wide<NW, V><<<blocks, 256, 0, st>>>(a);
-  else k_segsort_warp<NW, V><<<blocks, 256, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_after(a.n_items < kEarlyRows, wide && NW <= 16 ? k_segsort_warp_wide<NW, V> : k_segsort_warp<NW, V>, dim3(blocks), 256, 0, st, a);
   if (e != cudaSuccess) return e;
   // (the CTAs take groups off the lists as they go; small collections have few,
   // and CTAs that find none still cost their launch: 8.9 + 4.7 us of 1M suffixes

@@ -41,6 +41,7 @@ __device__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* scratch /*[blockD
 __global__ void __launch_bounds__(kCountThreads) k_poscount(const ReadIndex R, uint32_t n_reads, uint32_t q_max,
                                                             uint32_t* __restrict__ P) {
   extern __shared__ uint32_t sP[];
+  grid_launch_dependents();
   const uint32_t q0 = blockIdx.y * kSlab;
   const uint32_t qn = min(uint32_t(kSlab), q_max - q0);
   for (uint32_t x = threadIdx.x; x < qn * kRadix; x += blockDim.x) sP[x] = 0u;
@@ -65,15 +66,17 @@ __global__ void __launch_bounds__(kCountThreads) k_poscount(const ReadIndex R, u
   }
 }
 
-__global__ void __launch_bounds__(kRadix) k_digitbase(const uint32_t* __restrict__ P, uint32_t q_max, int uniform,
+__global__ void __launch_bounds__(kRadix) k_digitbase(const uint32_t* P, uint32_t q_max, int uniform,
                                                       uint32_t n_reads, uint32_t uniform_len,
                                                       const uint32_t* __restrict__ lenhist, uint32_t* __restrict__ base) {
   __shared__ unsigned long long s_z[kRadix / 32];
   __shared__ uint32_t s_scan[kRadix / 32];
+  grid_dependency_wait();
+  grid_launch_dependents();
   const uint32_t d = blockIdx.x, v = threadIdx.x;
   const uint32_t lo = 4u * d;
   uint32_t h = 0;
-  for (uint32_t q = lo; q < q_max; ++q) h += P[uint64_t(q) * kRadix + v];
+  for (uint32_t q = lo; q < q_max; ++q) h += __ldcg(P + uint64_t(q) * kRadix + v);
   // Z_d: suffixes whose digit d is entirely padding.
   unsigned long long z = 0;
   if (uniform) {
@@ -289,8 +292,7 @@ cudaError_t launch_poscount(const ReadIndex& R, uint32_t n_reads, uint32_t q_max
 cudaError_t launch_digitbase(const uint32_t* P, uint32_t q_max, uint32_t D, int uniform, uint32_t n_reads,
                              uint32_t uniform_len, const uint32_t* lenhist, uint32_t* base, cudaStream_t st) {
   if (D == 0) return cudaSuccess;
-  k_digitbase<<<D, kRadix, 0, st>>>(P, q_max, uniform, n_reads, uniform_len, lenhist, base);
-  return cudaGetLastError();
+  return launch_after(true, k_digitbase, dim3(D), kRadix, 0, st, P, q_max, uniform, n_reads, uniform_len, lenhist, base);
 }
 
 cudaError_t launch_identity(const ReadIndex& R, uint32_t n_reads, void* vals, int id_bytes, cudaStream_t st) {

@@ -44,9 +44,6 @@
 namespace cxbwt {
 namespace {
 
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // The m <= 16 bases of a read that end at its position `end` (the base at
 // end - 1 in the low two bits, the one before it above, ...).
 __device__ __forceinline__ uint32_t bases_before(const ReadIndex& R, uint64_t off, uint32_t end) {
@@ -750,16 +747,7 @@ __global__ void __launch_bounds__(kMergeThreads, kMergeBlocks) k_merge_step(cons
 
 template <int K, bool WIDE, bool LAST>
 cudaError_t launch_step(const MergeArgs& a, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.n_tiles);
-  cfg.blockDim = dim3(kMergeThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_merge_step<K, WIDE, LAST>, a);
+  return launch_after(true, k_merge_step<K, WIDE, LAST>, dim3(a.n_tiles), kMergeThreads, 0, st, a);
 }
 
 }  // namespace

@@ -50,7 +50,8 @@ constexpr uint64_t kOffVals1 = align256(kOffVals0 + kMaxRows * 4);
 constexpr uint64_t kOffKeys0 = align256(kOffVals1 + kMaxRows * 4);
 constexpr uint64_t kOffKeys1 = align256(kOffKeys0 + kMaxRows * 4);
 constexpr uint64_t kOffStatus = align256(kOffKeys1 + kMaxRows * 4);
-constexpr uint64_t kOffP = align256(kOffStatus + kMaxTiles * kRadix * 8);
+constexpr uint64_t kOffMisc = align256(kOffStatus + kMaxTiles * kRadix * 8);  // and kOffP: cleared together
+constexpr uint64_t kOffP = kOffMisc + 256;
 constexpr uint64_t kOffBase = align256(kOffP + uint64_t(kMaxLen) * kRadix * 4);
 // Reads of at most kMaxLen bases finish their groups with keys of at most
 // 16 words (segsort_words), which sets the CTA size of the group finish.
@@ -62,10 +63,9 @@ constexpr uint64_t kCtaCap = cta_list_cap(kMaxRows), kBigCap = big_list_cap(kMax
 constexpr uint32_t kEpochsPerCall = uint32_t(4 + 4 * kMaxW * kBigCap);
 constexpr uint64_t kOffSeg = align256(kOffBase + uint64_t(kMaxD + 5) * kRadix * 4);
 constexpr uint64_t kOffRhist = align256(kOffSeg + (kCtaCap + kBigCap) * 8);
-constexpr uint64_t kOffMisc = align256(kOffRhist + uint64_t(kMaxW) * 4 * kRadix * 4);
 // misc: [0] tile counter, [4] error word, [64] 5 x u64 counts, [128] 5 x u32 group-finish counters
 constexpr uint64_t kMiscSegAt = 128, kReadBack = kMiscSegAt + 8;
-constexpr uint64_t kNoallocScratchBytes = align256(kOffMisc + 256);
+constexpr uint64_t kNoallocScratchBytes = align256(kOffRhist + uint64_t(kMaxW) * 4 * kRadix * 4);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratchBytes];
 
@@ -139,8 +139,7 @@ extern "C" int cxbwt_build_noalloc(const uint32_t* reads_2bit, uint64_t n_reads,
   auto* d_counts = reinterpret_cast<unsigned long long*>(misc + 64);
   auto* d_seg = reinterpret_cast<uint32_t*>(misc + kMiscSegAt);
   // The previous call's contents stay in the array: clear what must start at zero.
-  NA_CUDA(cudaMemsetAsync(misc, 0, 256, st));
-  NA_CUDA(cudaMemsetAsync(base + kOffP, 0, uint64_t(L) * kRadix * 4, st));
+  NA_CUDA(cudaMemsetAsync(misc, 0, kOffP - kOffMisc + uint64_t(L) * kRadix * 4, st));
 
   const uint32_t shift = bits_for(L);
   const uint64_t n_words = (sum + 15) / 16;

@@ -97,6 +97,8 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) k_onesweep(const PassArgs
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < WARPS * kRadix; i += THREADS) (&s_whist[0][0])[i] = 0u;
   for (int i = tid; i < kRadix; i += THREADS) s_thist[i] = 0u;
+  grid_dependency_wait();
+  grid_launch_dependents();
   if (MODE == kSrcCollection)
     for (uint32_t i = tid; i <= a.n_coll; i += THREADS) s_coll[i] = a.coll_start[i];
   if (SPLIT)
@@ -424,7 +426,7 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) k_onesweep(const PassArgs
         // (after a wait that ran out, `before` is short: the outputs are then
         // unspecified but every write stays in bounds, and the error word says so)
       }
-      s_gbase[tid] = __ldg(a.digit_base + tid) + before - local_excl;
+      s_gbase[tid] = __ldcg(a.digit_base + tid) + before - local_excl;
     }
 
     // ---- 5. write out the staged tile ----------------------------------------
@@ -517,8 +519,7 @@ cudaError_t launch_mode(const PassArgs& a, cudaStream_t st) {
   if (MODE == kSrcCarried && a.prefetch && (reinterpret_cast<uintptr_t>(a.keys_in) & 15u) == 0 &&
       (reinterpret_cast<uintptr_t>(a.vals_in) & 15u) == 0)
     b.prefetch = grid_resident;
-  kern<<<a.n_tiles, S::threads, smem, st>>>(b);
-  return cudaGetLastError();
+  return launch_after(b.look_wide != 0, kern, dim3(a.n_tiles), S::threads, smem, st, b);
 }
 
 template <class V, class S>
