@@ -807,7 +807,36 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   // The merge plan sorts no slices.
   bool merged = !out_sa && !part && merge_pays(c, pl, false, pl.N) &&
                 pl.N <= ((c->opt.plan_flags & CXBWT_PLAN_MERGE) ? m1_bytes : m1) && merge_fits(c, pl, out_more);
-  if ((pl.N <= m1 || merged) && !part) {
+  // A part whose bucket counts are given and that fits one slice needs no more
+  // of them than the sums before, in and after it.
+  bool one_slice = false;
+  if (part && part->given_counts && !counts_only && pl.groups) {
+    const uint64_t* bc = part->given_counts;
+    auto sum = [&](size_t lo, size_t hi) {
+      uint64_t t = 0;
+      for (size_t b = lo; b < hi; ++b) t += bc[b];
+      return t;
+    };
+    part_row0 = sum(0, part->lo);
+    part_rows = sum(part->lo, part->hi);
+    const uint64_t total = part_row0 + part_rows + sum(part->hi, size_t(1) << kBucketBits);
+    if (total != pl.N)
+      return fail(c, CXBWT_EINVAL, "bucket counts sum to %llu, not the collection's %llu suffixes",
+                  (unsigned long long)total, (unsigned long long)pl.N);
+    one_slice = part_rows <= m1;
+  }
+  if (one_slice) {
+    r.bucket_bits = kBucketBits;
+    if (part_rows) {
+      Slice sl;
+      sl.whole = false;
+      sl.key_lo = uint32_t(uint64_t(part->lo) << (32 - kBucketBits));
+      sl.key_hi = uint64_t(part->hi) << (32 - kBucketBits);
+      sl.rows = uint32_t(part_rows);
+      sl.row0 = part_row0;
+      slices.push_back(sl);
+    }
+  } else if ((pl.N <= m1 || merged) && !part) {
     Slice sl;
     sl.rows = uint32_t(pl.N);
     slices.push_back(sl);
@@ -847,12 +876,7 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     }
     if (bh.empty() && part && part->given_counts) {
       r.bucket_bits = kBucketBits;
-      bh.assign(part->given_counts, part->given_counts + (size_t(1) << kBucketBits));
-      uint64_t total = 0;
-      for (uint64_t x : bh) total += x;
-      if (total != pl.N)
-        return fail(c, CXBWT_EINVAL, "bucket counts sum to %llu, not the collection's %llu suffixes",
-                    (unsigned long long)total, (unsigned long long)pl.N);
+      bh.assign(part->given_counts, part->given_counts + (size_t(1) << kBucketBits));  // (their sum is checked above)
     }
     if (bh.empty()) {
       r.bucket_bits = kBucketBits;
@@ -949,6 +973,8 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
       if (total != pl.N) return fail(c, CXBWT_EINTERNAL, "bucket counts sum to %llu, not N", (unsigned long long)total);
     }
     if (!part && r.bucket_bits == 8 && !refined) r.P_host = &P_host;
+  }
+  if (part || !slices[0].whole) {
     // The listing kernel where it can be used, also with the store in L2: it
     // lists 101M suffixes in 0.5 ms where generating and filtering them in
     // digit order took 0.9, and one digit pass more sorts only what was kept
