@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "group.cuh"
 
@@ -139,6 +140,97 @@ __device__ __forceinline__ uint32_t lex_less_mask(const uint32_t (&x)[NW], uint3
   for (int k = 0; k + 8 <= PP; k += 8) b = sub_borrow<8>(b, a + k, c + k);
   if (PP % 8) b = sub_borrow<4>(b, a + PP / 8 * 8, c + PP / 8 * 8);
   return b;
+}
+
+// The same with no padding, for the widths that compare in pairs below:
+// word_borrow<K> does K words (x[K - 1] first) after a word below them, x0 - y0;
+// (0, mask) continues a chain.
+template <int K>
+__device__ __forceinline__ uint32_t word_borrow(uint32_t x0, uint32_t y0, const uint32_t* x, const uint32_t* y);
+
+template <>
+__device__ __forceinline__ uint32_t word_borrow<8>(uint32_t x0, uint32_t y0, const uint32_t* x, const uint32_t* y) {
+  uint32_t r;
+  asm("{\n\t.reg .u32 t;\n\t"
+      "sub.cc.u32 t, %1, %2;\n\t"
+      "subc.cc.u32 t, %3, %4;\n\t"
+      "subc.cc.u32 t, %5, %6;\n\t"
+      "subc.cc.u32 t, %7, %8;\n\t"
+      "subc.cc.u32 t, %9, %10;\n\t"
+      "subc.cc.u32 t, %11, %12;\n\t"
+      "subc.cc.u32 t, %13, %14;\n\t"
+      "subc.cc.u32 t, %15, %16;\n\t"
+      "subc.cc.u32 t, %17, %18;\n\t"
+      "subc.u32 %0, 0, 0;\n\t}"
+      : "=r"(r)
+      : "r"(x0), "r"(y0), "r"(x[7]), "r"(y[7]), "r"(x[6]), "r"(y[6]), "r"(x[5]), "r"(y[5]), "r"(x[4]), "r"(y[4]),
+        "r"(x[3]), "r"(y[3]), "r"(x[2]), "r"(y[2]), "r"(x[1]), "r"(y[1]), "r"(x[0]), "r"(y[0]));
+  return r;
+}
+
+template <>
+__device__ __forceinline__ uint32_t word_borrow<10>(uint32_t x0, uint32_t y0, const uint32_t* x, const uint32_t* y) {
+  uint32_t r;
+  asm("{\n\t.reg .u32 t;\n\t"
+      "sub.cc.u32 t, %1, %2;\n\t"
+      "subc.cc.u32 t, %3, %4;\n\t"
+      "subc.cc.u32 t, %5, %6;\n\t"
+      "subc.cc.u32 t, %7, %8;\n\t"
+      "subc.cc.u32 t, %9, %10;\n\t"
+      "subc.cc.u32 t, %11, %12;\n\t"
+      "subc.cc.u32 t, %13, %14;\n\t"
+      "subc.cc.u32 t, %15, %16;\n\t"
+      "subc.cc.u32 t, %17, %18;\n\t"
+      "subc.cc.u32 t, %19, %20;\n\t"
+      "subc.cc.u32 t, %21, %22;\n\t"
+      "subc.u32 %0, 0, 0;\n\t}"
+      : "=r"(r)
+      : "r"(x0), "r"(y0), "r"(x[9]), "r"(y[9]), "r"(x[8]), "r"(y[8]), "r"(x[7]), "r"(y[7]), "r"(x[6]), "r"(y[6]),
+        "r"(x[5]), "r"(y[5]), "r"(x[4]), "r"(y[4]), "r"(x[3]), "r"(y[3]), "r"(x[2]), "r"(y[2]), "r"(x[1]), "r"(y[1]),
+        "r"(x[0]), "r"(y[0]));
+  return r;
+}
+
+template <>
+__device__ __forceinline__ uint32_t word_borrow<12>(uint32_t x0, uint32_t y0, const uint32_t* x, const uint32_t* y) {
+  uint32_t r;
+  asm("{\n\t.reg .u32 t;\n\t"
+      "sub.cc.u32 t, %1, %2;\n\t"
+      "subc.cc.u32 t, %3, %4;\n\t"
+      "subc.cc.u32 t, %5, %6;\n\t"
+      "subc.cc.u32 t, %7, %8;\n\t"
+      "subc.cc.u32 t, %9, %10;\n\t"
+      "subc.cc.u32 t, %11, %12;\n\t"
+      "subc.cc.u32 t, %13, %14;\n\t"
+      "subc.cc.u32 t, %15, %16;\n\t"
+      "subc.cc.u32 t, %17, %18;\n\t"
+      "subc.cc.u32 t, %19, %20;\n\t"
+      "subc.cc.u32 t, %21, %22;\n\t"
+      "subc.cc.u32 t, %23, %24;\n\t"
+      "subc.cc.u32 t, %25, %26;\n\t"
+      "subc.u32 %0, 0, 0;\n\t}"
+      : "=r"(r)
+      : "r"(x0), "r"(y0), "r"(x[11]), "r"(y[11]), "r"(x[10]), "r"(y[10]), "r"(x[9]), "r"(y[9]), "r"(x[8]),
+        "r"(y[8]), "r"(x[7]), "r"(y[7]), "r"(x[6]), "r"(y[6]), "r"(x[5]), "r"(y[5]), "r"(x[4]), "r"(y[4]), "r"(x[3]),
+        "r"(y[3]), "r"(x[2]), "r"(y[2]), "r"(x[1]), "r"(y[1]), "r"(x[0]), "r"(y[0]));
+  return r;
+}
+
+// ~0u if (x words, x0) < (y words, y0), NW = 10, 12, 16, 20, 24 or 32.
+template <int NW>
+__device__ __forceinline__ uint32_t pair_less_mask(const uint32_t (&x)[NW], uint32_t x0, const uint32_t (&y)[NW], uint32_t y0) {
+  // Chains of at most 12 words (27 operands), the least significant first.
+  constexpr int LOW = NW <= 12 ? NW : NW == 16 || NW == 32 ? 8 : NW / 2;
+  uint32_t b = word_borrow<LOW>(x0, y0, x + (NW - LOW), y + (NW - LOW));
+  if constexpr (NW == 32) b = word_borrow<12>(0u, b, x + 12, y + 12);
+  constexpr int TOP = NW == 32 ? 12 : NW - LOW;
+  if constexpr (TOP > 0) b = word_borrow<TOP>(0u, b, x, y);
+  return b;
+}
+
+__device__ __forceinline__ void count_unless(uint32_t* p, uint32_t mask) {  // *p += 1 in shared memory if mask is 0
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %1, 0;\n\t@p red.shared.add.u32 [%0], 1;\n\t}"
+               ::"r"(uint32_t(__cvta_generic_to_shared(p))), "r"(mask) : "memory");
 }
 
 template <class V>
@@ -258,6 +350,95 @@ __device__ void warp_rank_window(const SegArgs& a, uint32_t cur, uint32_t n_rows
   __syncwarp();  // the next window reuses the shared rows
 }
 
+// The same for windows of 32 rows of 10 or more words, where the subtractions
+// bound the kernel (ALU 83% busy): each pair of rows of a group is compared
+// once.  A row compares itself with the g / 2 rows after it (around the group's
+// end), counts those that order before it, and adds one to the counters of the
+// others.  60M rows of 150-base reads 1,627 -> 1,551 us, a build of 48M of 20 to
+// 300 bases 4.90 -> 4.66 ms; with 6 words (100 bases) no faster, and windows of
+// 64 rows lost by it (505M rows in three slices 33.8 -> 34.8 ms).  Up to 20 words
+// a group's rows are in shared memory twice in a row, so that the rows after one
+// are consecutive.
+template <int NW>
+struct PairRows {
+  static constexpr int Q = (NW + 3) / 4;        // uint4 per row, each in a plane of its own: no bank conflicts
+  static constexpr bool TWICE = Q <= 5;         // (with six, eight warps' rows would pass 48 KB)
+  static constexpr int SLOTS = TWICE ? 64 : 32;
+  uint4 r[Q][SLOTS];
+  uint32_t before[SLOTS];                       // members found to be before the row by their own comparisons
+};
+
+template <int NW, class V>
+__device__ void warp_rank_pairs(const SegArgs& a, uint32_t cur, uint32_t n_rows, uint32_t heads, int lane, PairRows<NW>& sw) {
+  constexpr int Q = PairRows<NW>::Q;
+  constexpr bool TWICE = PairRows<NW>::TWICE;
+  V* vals = static_cast<V*>(a.vals);
+  const uint32_t row = uint32_t(lane);
+  // The row's group [g0, ge), of g rows (0 past the window's end).
+  const uint32_t upto = heads & (row == 31 ? ~0u : (2u << row) - 1), after = heads & ~upto;
+  const uint32_t g0 = 31 - __clz(upto);
+  const uint32_t ge = after ? min(uint32_t(__ffs(after)) - 1, n_rows) : n_rows;
+  const uint32_t g = row < n_rows ? ge - g0 : 0u;
+  const uint32_t slot = TWICE ? g0 + row : row;
+  V v = 0;
+  uint32_t mine[NW];
+  if (g > 1) {
+    v = vals[cur + row];
+    gather_words<NW>(a.R, decode(a.R, v), a.depth, mine);
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const uint4 w = make_uint4(mine[4 * q], mine[4 * q + 1], 4 * q + 2 < NW ? mine[4 * q + 2] : 0u,
+                                 4 * q + 3 < NW ? mine[4 * q + 3] : 0u);
+      sw.r[q][slot] = w;
+      if (TWICE) sw.r[q][slot + g] = w;
+    }
+    sw.before[slot] = 0u;
+    if (TWICE) sw.before[slot + g] = 0u;
+  }
+  __syncwarp();
+  // The next (g - 1) / 2 rows, and for half the rows of an even group the one
+  // across: every pair once.
+  const uint32_t n_cmp = g > 1 ? (g - 1) / 2 + ((g & 1) == 0 && row - g0 < g / 2 ? 1u : 0u) : 0u;
+  const uint32_t to_end = ge - row - 1;  // rows of the group after this one
+  uint32_t rank = 0;
+  for (uint32_t t = 1; t <= n_cmp; ++t) {
+    const uint32_t src = TWICE ? slot + t : slot + t - (t > to_end ? g : 0u);
+    uint32_t ov[NW];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      const uint4 o = sw.r[q][src];
+      ov[4 * q] = o.x;
+      ov[4 * q + 1] = o.y;
+      if (4 * q + 2 < NW) ov[4 * q + 2] = o.z;
+      if (4 * q + 3 < NW) ov[4 * q + 3] = o.w;
+    }
+    // That row orders before this one: smaller words, or equal words and an
+    // earlier row (one past the group's end, counted around it).
+    const uint32_t less = pair_less_mask<NW>(ov, to_end, mine, t);
+    rank -= less;  // ~0u is -1
+    count_unless(&sw.before[src], less);
+  }
+  __syncwarp();  // every counter is complete, every row read
+  if (g > 1) {
+    const uint32_t to = g0 + rank + sw.before[slot] + (TWICE ? sw.before[slot + g] : 0u);
+    if (to != row) vals[cur + to] = v;
+  }
+  __syncwarp();  // the next window reuses the shared rows
+}
+
+// Rows of a warp's window, and the function that ranks them.
+template <int NW, int SPAN>
+struct Window {
+  static constexpr bool PAIRS = SPAN == 32 && NW >= 10;
+  using Rows = typename std::conditional<PAIRS, PairRows<NW>, RowWords<NW, SPAN>>::type;
+  template <class V>
+  static __device__ __forceinline__ void rank(const SegArgs& a, uint32_t cur, uint32_t n_rows, typename Heads<SPAN>::T heads,
+                                              int lane, Rows& sw) {
+    if constexpr (PAIRS) warp_rank_pairs<NW, V>(a, cur, n_rows, heads, lane, sw);
+    else warp_rank_window<NW, SPAN, V>(a, cur, n_rows, heads, lane, sw);
+  }
+};
+
 // First row r >= from (r < n) whose window differs from row r-1, or n.
 __device__ uint32_t next_head(const SegArgs& a, uint32_t from, int lane) {
   if (from >= a.n_items) return a.n_items;
@@ -282,7 +463,8 @@ __device__ uint32_t next_head(const SegArgs& a, uint32_t from, int lane) {
 // Finish one group of more than SPAN rows [gs, ge): skip its finished
 // prefix, sort a remainder of at most SPAN rows here, list a larger one.
 template <int NW, int SPAN, class V>
-__device__ void finish_long_group(const SegArgs& a, uint32_t gs, uint32_t ge, int lane, RowWords<NW, SPAN>& sw) {
+__device__ void finish_long_group(const SegArgs& a, uint32_t gs, uint32_t ge, int lane,
+                                  typename Window<NW, SPAN>::Rows& sw) {
   const V* vals = static_cast<const V*>(a.vals);
   uint32_t lo = gs, hi = ge;
   while (lo < hi) {
@@ -292,7 +474,7 @@ __device__ void finish_long_group(const SegArgs& a, uint32_t gs, uint32_t ge, in
   const uint32_t m = ge - lo;
   if (m < 2) return;
   if (m <= uint32_t(SPAN)) {
-    warp_rank_window<NW, SPAN, V>(a, lo, m, typename Heads<SPAN>::T(1), lane, sw);
+    Window<NW, SPAN>::template rank<V>(a, lo, m, typename Heads<SPAN>::T(1), lane, sw);
   } else if (lane == 0) {
     // Up to kSmallCta rows: cta_list from the front (counts[0]); up to
     // CtaRows: cta_list from the back (counts[3]; the two never meet, as each
@@ -321,10 +503,11 @@ template <int NW, class V, int SPAN>
 __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
   using H = typename Heads<SPAN>::T;
   const int lane = threadIdx.x & 31;
-  __shared__ RowWords<NW, SPAN> s_rows[8];
+  using Rows = typename Window<NW, SPAN>::Rows;
+  __shared__ Rows s_rows[8];
   grid_dependency_wait();
   grid_launch_dependents();
-  RowWords<NW, SPAN>& sw = s_rows[threadIdx.x >> 5];
+  Rows& sw = s_rows[threadIdx.x >> 5];
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t chunk = a.chunk, n_chunks = (a.n_items + chunk - 1) / chunk;
   for (uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_chunks; c += warps) {
@@ -355,7 +538,7 @@ __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
       const H heads = (hm << 1) | H(1);
       // A window of only one-row groups is already sorted.
       const H full = n_rows == uint32_t(SPAN) ? ~H(0) : ((H(1) << n_rows) - 1);
-      if ((heads & full) != full) warp_rank_window<NW, SPAN, V>(a, cur, n_rows, heads, lane, sw);
+      if ((heads & full) != full) Window<NW, SPAN>::template rank<V>(a, cur, n_rows, heads, lane, sw);
       cur += n_rows;
     }
   }
@@ -525,7 +708,10 @@ cudaError_t launch_nw(const SegArgs& args, int sm_count, bool wide, cudaStream_t
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
   // Rows of the widest keys (long reads) would not fit twice in shared memory.
-  cudaError_t e = launch_after(a.n_items < kEarlyRows, wide && NW <= 16 ? k_segsort_warp_wide<NW, V> : k_segsort_warp<NW, V>, dim3(blocks), 256, 0, st, a);
+  auto kern = k_segsort_warp<NW, V>;
+  if constexpr (NW <= 16)
+    if (wide) kern = k_segsort_warp_wide<NW, V>;
+  cudaError_t e = launch_after(a.n_items < kEarlyRows, kern, dim3(blocks), 256, 0, st, a);
   if (e != cudaSuccess) return e;
   // (the CTAs take groups off the lists as they go; small collections have few,
   // and CTAs that find none still cost their launch: 8.9 + 4.7 us of 1M suffixes
