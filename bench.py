@@ -292,6 +292,9 @@ def phase_rates(st, steps, n_reads, bases, idb, peak):
       written;
     * emission: the id of every suffix read, its 2-bit symbol written, 8 B per
       $ row, the read store (a quarter byte per base) read once;
+    * merge steps (builds that the merge plan took; nothing is sorted then): at
+      each of L + 1 steps the rows so far (2 bits, read and written) and 12
+      bytes per read (read and written);
     * histograms and planning (the rest of the build): the read store and the
       read lengths read once.
 
@@ -301,7 +304,8 @@ def phase_rates(st, steps, n_reads, bases, idb, peak):
     sort_ms = st["sort_pass_ms"] / steps
     group_ms = st["group_ms"] / steps
     emit_ms = st["emit_ms"] / steps
-    rest_ms = st["build_ms"] / steps - sort_ms - group_ms - emit_ms
+    merge_ms = st.get("merge_ms", 0.0) / steps
+    rest_ms = st["build_ms"] / steps - sort_ms - group_ms - emit_ms - merge_ms
     carried_ms = st["carried_pass_ms"] / steps
     gen_items = (st["sort_pass_items"] - st["carried_pass_items"]) / steps
     slices = st["slices"] / steps
@@ -314,6 +318,7 @@ def phase_rates(st, steps, n_reads, bases, idb, peak):
              "generating_passes": (sort_ms - carried_ms, (4 + idb) * gen_items + slices * bases / 4),
              "group_finish": (group_ms, (4 + 2 * idb) * N),
              "emission": (emit_ms, idb * N + N / 4 + 8 * n_reads + bases / 4),
+             "merge_steps": (merge_ms, (N / n_reads) * (0.5 * N / 2 + 24 * n_reads)),
              "histograms_and_planning": (rest_ms, bases / 4 + 4 * n_reads)}
     out = {}
     for name, (ms, nbytes) in model.items():
