@@ -505,8 +505,6 @@ __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
   const int lane = threadIdx.x & 31;
   using Rows = typename Window<NW, SPAN>::Rows;
   __shared__ Rows s_rows[8];
-  grid_dependency_wait();
-  grid_launch_dependents();
   Rows& sw = s_rows[threadIdx.x >> 5];
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t chunk = a.chunk, n_chunks = (a.n_items + chunk - 1) / chunk;
@@ -546,6 +544,8 @@ __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
 
 template <int NW, class V>
 __global__ void __launch_bounds__(256) k_segsort_warp(const SegArgs a) {
+  grid_dependency_wait();
+  grid_launch_dependents();
   segsort_warp_body<NW, V, 32>(a);
 }
 
@@ -708,10 +708,11 @@ cudaError_t launch_nw(const SegArgs& args, int sm_count, bool wide, cudaStream_t
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
   // Rows of the widest keys (long reads) would not fit twice in shared memory.
+  // (The wide kernel is launched plainly: it serves stores out of L2.)
   auto kern = k_segsort_warp<NW, V>;
   if constexpr (NW <= 16)
     if (wide) kern = k_segsort_warp_wide<NW, V>;
-  cudaError_t e = launch_after(a.n_items < kEarlyRows, kern, dim3(blocks), 256, 0, st, a);
+  cudaError_t e = launch_after(!wide && a.n_items < kEarlyRows, kern, dim3(blocks), 256, 0, st, a);
   if (e != cudaSuccess) return e;
   // (the CTAs take groups off the lists as they go; small collections have few,
   // and CTAs that find none still cost their launch: 8.9 + 4.7 us of 1M suffixes
