@@ -473,10 +473,15 @@ class Context:
         _need(8, out_dollar_pos=out_dollar_pos, out_counts=out_counts)
         if _nbytes(out_words) < 4 * part_words(row0, rows):
             raise ValueError("out_words holds fewer words than the part needs")
+        words = out_words
+        if rows == 0 and _ptr(out_words) and _nbytes(out_words) < 4:
+            # An empty part has one word of zeros when row0 is inside a word;
+            # callers that merge nothing need not hold it.
+            words = np.zeros(1, dtype=np.uint32)
         r0, nr = ctypes.c_uint64(), ctypes.c_uint64()
         _check(lib().cxbwt_build_part(self._h, _ptr(reads_2bit), n, _ptr(lens), bucket_lo, bucket_hi,
                                       None if bc is None else bc.ctypes.data,
-                                      _ptr(out_words), _ptr(out_dollar_pos), _ptr(out_counts), ctypes.byref(r0),
+                                      _ptr(words), _ptr(out_dollar_pos), _ptr(out_counts), ctypes.byref(r0),
                                       ctypes.byref(nr), _stream_ptr(stream)), self._h)
         if (int(r0.value), int(nr.value)) != (row0, rows):
             raise CxbwtError(-7, f"part rows [{r0.value}, +{nr.value}) differ from the plan's [{row0}, +{rows})")

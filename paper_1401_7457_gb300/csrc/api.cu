@@ -1013,6 +1013,19 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     CX_CUDA(c, cudaMemsetAsync(r.d_dollar, 0xFF, n * 8, st));  // reads whose $ row is in another part
   }
 
+  if (part && !part_rows) {
+    // No suffix in the range: no plan runs.  The word that row0 lies in has no
+    // symbol of the part, and the part's counts are 0.
+    if (bwt_words) CX_CUDA(c, cudaMemsetAsync(r.d_bwt, 0, bwt_words * 4, st));
+    CX_CUDA(c, cudaMemsetAsync(r.d_counts, 0, 5 * 8, st));
+    if (c->opt.timing) CX_CUDA(c, cudaEventRecord(c->ev[0], st));
+    if (!bwt_dev && bwt_words) {
+      CX_CUDA(c, cudaMemcpyAsync(out_bwt, r.d_bwt, bwt_words * 4, cudaMemcpyDeviceToHost, st));
+      r.d2h += bwt_words * 4;
+    }
+    return finish_build(c, r, Outs{out_bwt, out_dollar, out_counts, out_sa, bwt_dev, dollar_dev, counts_dev, sa_dev}, h2d,
+                        0);
+  }
   if (part && merge_pays(c, pl, true, part_rows) && pl.N <= m1 && merge_fits(c, pl, 0)) merged = true;
   if (merged) {
     if (part) CX_CUDA(c, cudaMemsetAsync(r.d_counts, 0, 5 * 8, st));

@@ -1,0 +1,44 @@
+"""Edges of bucket-range parts: ranges that hold no suffix."""
+import numpy as np
+import pytest
+
+from paper_1401_7457_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def device(a):
+    return torch.from_numpy(a.view(np.int32)).cuda()
+
+
+@pytest.mark.parametrize("given", [True, False])
+@pytest.mark.parametrize("where", ["device", "host"])
+@pytest.mark.parametrize("length", [1, 10, 20, 100, 300])
+def test_empty_part(length, where, given):
+    """A range without suffixes whose first row is inside a word: that word is
+    written as 0, the counts as 0 and every $ row as ~0, whatever the buffers
+    (the caller's and the context's) held before; no plan runs for it."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    codes, lens = synth.uniform_reads(1001, length, length)
+    words = binding.pack_codes(codes)
+    if where == "device":
+        words, lens = device(words), device(lens)
+    with binding.Context(device=0) as c:
+        c.build(words, lens)
+        counts = c.bucket_counts(words, lens)
+        before = np.concatenate([[0], np.cumsum(counts.astype(np.int64))])
+        lo = int(np.nonzero((counts == 0) & (before[:-1] % 16 != 0))[0][0])
+        row0 = int(before[lo])
+        out = np.full(1, 0xFFFFFFFF, dtype=np.uint32), np.full(1001, 7, dtype=np.uint64), np.full(5, 7, dtype=np.uint64)
+        if where == "device":
+            out = device(out[0]), torch.full((1001,), 7, device="cuda"), torch.full((5,), 7, device="cuda")
+        c.reset_stats()
+        c.build_part(words, lens, lo, lo + 1, row0, 0, *out, bucket_counts=counts if given else None)
+        if where == "device":
+            out = [t.cpu().numpy() for t in out]
+        assert int(out[0][0]) == 0
+        assert (out[1].view(np.uint64) == np.uint64(0xFFFFFFFFFFFFFFFF)).all() and not out[2].any()
+        assert c.stats()["merge_launches"] == 0 and c.stats()["sort_pass_launches"] == 0
