@@ -494,7 +494,7 @@ struct Outs {
 
 // The end of a build whose kernels and BWT copies are enqueued: the other
 // outputs' copies, the wait, the statistics (of n_sorted sorted slices: none
-// when the merge plan built it).
+// when the merge plan built it, or for a part without suffixes).
 static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_t n_sorted) {
   const Plan& pl = r.pl;
   cudaStream_t st = r.st;
@@ -543,7 +543,7 @@ static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_
   c->stats.h2d_bytes += h2d;
   c->stats.d2h_bytes += r.d2h;
   c->stats.device_bytes_held = c->held;
-  c->stats.slices += std::max<size_t>(n_sorted, 1);
+  c->stats.slices += r.merge_launches ? 1 : n_sorted;
   c->stats.carried_pass_launches += r.carried_launches;
   c->stats.carried_pass_items += r.carried_items;
   c->stats.merge_launches += r.merge_launches;
@@ -576,7 +576,7 @@ static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_
       else c->stats.sort_pass_ms += ms;  // the split pass runs before every slice
     }
     c->stats.build_ms += ms_all;
-    if (!n_sorted) c->stats.merge_ms += ms_all;
+    if (r.merge_launches) c->stats.merge_ms += ms_all;
   }
   c->stats.builds += 1;
   c->stats.bases += pl.sum;

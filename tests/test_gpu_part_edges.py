@@ -42,3 +42,21 @@ def test_empty_part(length, where, given):
         assert int(out[0][0]) == 0
         assert (out[1].view(np.uint64) == np.uint64(0xFFFFFFFFFFFFFFFF)).all() and not out[2].any()
         assert c.stats()["merge_launches"] == 0 and c.stats()["sort_pass_launches"] == 0
+
+
+@pytest.mark.parametrize("flags", [0, 64])
+def test_empty_part_counts_as_no_slice(flags):
+    """Nothing is sorted or merged for an empty part: its time is no plan's."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    codes, lens = synth.uniform_reads(1001, 50, 3)
+    words, lens = device(binding.pack_codes(codes)), device(lens)
+    with binding.Context(device=0, plan_flags=flags, timing=True) as c:
+        counts = c.bucket_counts(words, lens)
+        lo = int(np.nonzero(counts == 0)[0][0])
+        c.reset_stats()
+        c.build_part(words, lens, lo, lo + 1, int(counts[:lo].sum()), 0, bucket_counts=counts)
+        st = c.stats()
+        assert st["builds"] == 1 and st["slices"] == 0 and st["build_ms"] > 0
+        assert st["merge_ms"] == 0 and st["merge_launches"] == 0
