@@ -693,7 +693,6 @@ cudaError_t launch_cta_nw(const SegArgs& a, uint32_t grid, const uint2* list, co
     configured.fetch_or(bit, std::memory_order_release);
   }
   return launch_after(a.n_items < kEarlyRows, kern, dim3(grid), THREADS, smem, st, a, list, n_ptr, cap, dir, work);
-  return cudaGetLastError();
 }
 
 // The warp kernel, then the small-group and the large-group CTA kernels over
