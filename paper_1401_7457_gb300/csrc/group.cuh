@@ -35,7 +35,6 @@ struct SegArgs {
   uint32_t* counts;       // zero on entry: [0] small remainders (cta_list front), [1] big_list length,
                           // [2] small work counter, [3] larger CTA remainders (cta_list back), [4] their work counter
   uint32_t* err;
-  uint32_t chunk;         // rows a warp scans at a time (set by the launch)
 };
 
 // Key words a group remainder is sorted by for reads of at most max_len bases

@@ -216,11 +216,11 @@ __device__ __forceinline__ uint32_t word_borrow<12>(uint32_t x0, uint32_t y0, co
   return r;
 }
 
-// ~0u if (x words, x0) < (y words, y0), NW = 10, 12, 16, 20, 24 or 32.
+// ~0u if (x words, x0) < (y words, y0), NW = 10, 12, 16, 20 or 32.
 template <int NW>
 __device__ __forceinline__ uint32_t pair_less_mask(const uint32_t (&x)[NW], uint32_t x0, const uint32_t (&y)[NW], uint32_t y0) {
   // Chains of at most 12 words (27 operands), the least significant first.
-  constexpr int LOW = NW <= 12 ? NW : NW == 16 || NW == 32 ? 8 : NW / 2;
+  constexpr int LOW = NW <= 12 ? NW : NW == 20 ? 10 : 8;
   uint32_t b = word_borrow<LOW>(x0, y0, x + (NW - LOW), y + (NW - LOW));
   if constexpr (NW == 32) b = word_borrow<12>(0u, b, x + 12, y + 12);
   constexpr int TOP = NW == 32 ? 12 : NW - LOW;
@@ -354,15 +354,22 @@ __device__ void warp_rank_window(const SegArgs& a, uint32_t cur, uint32_t n_rows
 // bound the kernel (ALU 83% busy): each pair of rows of a group is compared
 // once.  A row compares itself with the g / 2 rows after it (around the group's
 // end), counts those that order before it, and adds one to the counters of the
-// others.  60M rows of 150-base reads 1,627 -> 1,551 us, a build of 48M of 20 to
-// 300 bases 4.90 -> 4.66 ms; with 6 words (100 bases) no faster, and windows of
-// 64 rows lost by it (505M rows in three slices 33.8 -> 34.8 ms).  Up to 20 words
-// a group's rows are in shared memory twice in a row, so that the rows after one
-// are consecutive.
+// others.  A collection without groups (unrelated reads) pays for it in resident
+// warps, so the widths and their registers are those that lose little there.
+// Builds by this plan, pairs compared twice / once, reads of a 20x genome and
+// unrelated reads: 400k of 150 bases (10 words) 3,391 / 3,298 and 2,374 / 2,432
+// us; 200k of 200 (12) 2,522 / 2,362 and 1,701 / 1,686; 200k of 250 (16) 3,671 /
+// 3,156 and 2,138 / 2,099; 200k of 300 (20, 24 before) 4,931 / 4,182 and 2,607 /
+// 2,559; 100k of 500 (32) 7,200 / 4,699 and 2,624 / 2,584.  Not with 24 words:
+// 150k of 400 bases 5,045 / 4,633, but 2,666 / 2,775; nor with 6 (no faster), nor
+// in windows of 64 rows (505M rows in three slices 33.8 -> 34.8 ms).  With 12 and
+// 16 words a group's rows are in shared memory twice in a row, so that the rows
+// after one are consecutive; with the other widths that costs more L1 than it
+// saves.
 template <int NW>
 struct PairRows {
   static constexpr int Q = (NW + 3) / 4;        // uint4 per row, each in a plane of its own: no bank conflicts
-  static constexpr bool TWICE = Q <= 5;         // (with six, eight warps' rows would pass 48 KB)
+  static constexpr bool TWICE = NW == 12 || NW == 16;
   static constexpr int SLOTS = TWICE ? 64 : 32;
   uint4 r[Q][SLOTS];
   uint32_t before[SLOTS];                       // members found to be before the row by their own comparisons
@@ -429,7 +436,7 @@ __device__ void warp_rank_pairs(const SegArgs& a, uint32_t cur, uint32_t n_rows,
 // Rows of a warp's window, and the function that ranks them.
 template <int NW, int SPAN>
 struct Window {
-  static constexpr bool PAIRS = SPAN == 32 && NW >= 10;
+  static constexpr bool PAIRS = SPAN == 32 && NW >= 10 && NW != 24;
   using Rows = typename std::conditional<PAIRS, PairRows<NW>, RowWords<NW, SPAN>>::type;
   template <class V>
   static __device__ __forceinline__ void rank(const SegArgs& a, uint32_t cur, uint32_t n_rows, typename Heads<SPAN>::T heads,
@@ -492,14 +499,14 @@ __device__ void finish_long_group(const SegArgs& a, uint32_t gs, uint32_t ge, in
   }
 }
 
-// Each warp owns the groups whose first row lies in its chunk of kChunk rows
+// Each warp owns the groups whose first row lies in its chunk of CHUNK rows
 // and walks them in windows of up to SPAN rows made of whole groups.  SPAN is
 // 64 (two rows per lane) when the read store is out of L2: the gathers of a
 // window then wait on DRAM, and a window of two rows per lane puts twice as
 // many in flight and spends fewer rounds on groups of 20 to 30 rows (reads at
 // tens-fold coverage); with the store in L2 the ranking's instructions
 // dominate and 32-row windows, with fewer of them, are faster (measured).
-template <int NW, class V, int SPAN>
+template <int NW, class V, int SPAN, uint32_t CHUNK>
 __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
   using H = typename Heads<SPAN>::T;
   const int lane = threadIdx.x & 31;
@@ -507,10 +514,10 @@ __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
   __shared__ Rows s_rows[8];
   Rows& sw = s_rows[threadIdx.x >> 5];
   const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-  const uint32_t chunk = a.chunk, n_chunks = (a.n_items + chunk - 1) / chunk;
+  const uint32_t n_chunks = a.n_items / CHUNK + (a.n_items % CHUNK ? 1 : 0);
   for (uint32_t c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < n_chunks; c += warps) {
-    const uint32_t limit = c + 1 < n_chunks ? (c + 1) * chunk : a.n_items;
-    uint32_t cur = next_head(a, c * chunk, lane);
+    const uint32_t limit = c + 1 < n_chunks ? (c + 1) * CHUNK : a.n_items;
+    uint32_t cur = next_head(a, c * CHUNK, lane);
     while (cur < limit) {
       // Heads among rows cur+1 .. cur+SPAN (bit r-1 for row cur+r); row
       // limit and beyond belong to the next chunk's groups, so the first
@@ -542,11 +549,20 @@ __device__ __forceinline__ void segsort_warp_body(const SegArgs& a) {
   }
 }
 
-template <int NW, class V>
-__global__ void __launch_bounds__(256) k_segsort_warp(const SegArgs a) {
+// CTAs per SM the registers are held to, where the compiler's own choice (0)
+// keeps fewer resident than the scan of a collection without groups needs:
+// 10 words 56 registers, 4 CTAs (400k unrelated reads of 150 bases: 2,480 us, 2,431
+// with five); 20 words 77, 3 (200k of 300 bases: 2,678, 2,576 with four).
+template <int NW>
+constexpr int warp_blocks() { return NW == 10 ? 5 : NW == 20 ? 4 : 0; }
+
+// CHUNK is compiled in: as a field of the arguments it cost 4 to 16 registers
+// in every width (8 words: 47 instead of 32).
+template <int NW, class V, uint32_t CHUNK>
+__global__ void __launch_bounds__(256, warp_blocks<NW>()) k_segsort_warp(const SegArgs a) {
   grid_dependency_wait();
   grid_launch_dependents();
-  segsort_warp_body<NW, V, 32>(a);
+  segsort_warp_body<NW, V, 32, CHUNK>(a);
 }
 
 // The 64-row windows wait on DRAM gathers: resident warps hide that wait, so
@@ -557,7 +573,7 @@ __global__ void __launch_bounds__(256) k_segsort_warp(const SegArgs a) {
 constexpr int kWideBlocks = 6;
 template <int NW, class V>
 __global__ void __launch_bounds__(256, kWideBlocks) k_segsort_warp_wide(const SegArgs a) {
-  segsort_warp_body<NW, V, 64>(a);
+  segsort_warp_body<NW, V, 64, kChunk>(a);
 }
 
 // Shared-memory bitonic sort of one listed group per CTA, for groups of up to
@@ -698,17 +714,17 @@ cudaError_t launch_cta_nw(const SegArgs& a, uint32_t grid, const uint2* list, co
 // The warp kernel, then the small-group and the large-group CTA kernels over
 // the two ends of the list it fills.
 template <int NW, class V>
-cudaError_t launch_nw(const SegArgs& args, int sm_count, bool wide, cudaStream_t st) {
-  SegArgs a = args;
+cudaError_t launch_nw(const SegArgs& a, int sm_count, bool wide, cudaStream_t st) {
   const uint32_t cap = uint32_t(sm_count) * 16;
-  a.chunk = a.n_items / kSmallChunk <= 8 * cap ? kSmallChunk : kChunk;
-  const uint32_t n_chunks = (a.n_items + a.chunk - 1) / a.chunk;
+  if (NW > 16) wide = false;
+  const uint32_t chunk = !wide && a.n_items / kSmallChunk <= 8 * cap ? kSmallChunk : kChunk;
+  const uint32_t n_chunks = a.n_items / chunk + (a.n_items % chunk ? 1 : 0);
   uint32_t blocks = (n_chunks + 7) / 8;
   if (blocks > cap) blocks = cap;
   if (blocks == 0) blocks = 1;
   // Rows of the widest keys (long reads) would not fit twice in shared memory.
   // (The wide kernel is launched plainly: it serves stores out of L2.)
-  auto kern = k_segsort_warp<NW, V>;
+  auto kern = chunk == kSmallChunk ? k_segsort_warp<NW, V, kSmallChunk> : k_segsort_warp<NW, V, kChunk>;
   if constexpr (NW <= 16)
     if (wide) kern = k_segsort_warp_wide<NW, V>;
   cudaError_t e = launch_after(!wide && a.n_items < kEarlyRows, kern, dim3(blocks), 256, 0, st, a);
