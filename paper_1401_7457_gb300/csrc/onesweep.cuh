@@ -65,7 +65,16 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_256(uint32_t x, uint32_
   return warp_prefix + incl - x;
 }
 
-template <class V, int THREADS, int IPT, int MIN_BLOCKS, int MODE, bool WRITE_KEY, bool FILTER>
+// An id or key of the pass before.  A pass launched early starts while that pass
+// still writes them, so it may not use the read-only path, whose data must not
+// change while the kernel runs; the others do (__ldcg in every pass: 1 to 1.5% of
+// a build of 40M rows, plain loads 1%, a choice at run time 2.5%).
+template <bool EARLY, class T>
+__device__ __forceinline__ T load_input(const T* p) {
+  return EARLY ? __ldcg(p) : __ldg(p);
+}
+
+template <class V, int THREADS, int IPT, int MIN_BLOCKS, int MODE, bool WRITE_KEY, bool FILTER, bool EARLY>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) k_onesweep(const PassArgs a) {
   constexpr int TILE = THREADS * IPT;
   constexpr int WARPS = THREADS / 32;
@@ -204,14 +213,14 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) k_onesweep(const PassArgs
   #pragma unroll
       for (int j = 0; j < IPT; ++j) {
         const I idx = warp_base + j * 32;
-        val[j] = (!NINTH || idx < n_in) ? __ldg(vals_in + idx) : V(0);
+        val[j] = (!NINTH || idx < n_in) ? load_input<EARLY>(vals_in + idx) : V(0);
       }
     }
     if (CARRY_KEY) {
   #pragma unroll
       for (int j = 0; j < IPT; ++j) {
         const I idx = warp_base + j * 32;
-        key[j] = (!NINTH || idx < n_in) ? __ldg(a.keys_in + idx) : 0u;
+        key[j] = (!NINTH || idx < n_in) ? load_input<EARLY>(a.keys_in + idx) : 0u;
       }
     } else if (MODE == kSrcLength) {
   #pragma unroll
@@ -490,12 +499,18 @@ using Shape64x8 = Shape<256, 8, 5>;    // 2048 items (64-bit ids: 24 KB staged, 
 template <class V, class S, int MODE, bool WK, bool F>
 cudaError_t launch_mode(const PassArgs& a, cudaStream_t st) {
   const size_t smem = size_t(S::threads) * S::ipt * (sizeof(uint32_t) + sizeof(V));
-  auto kern = k_onesweep<V, S::threads, S::ipt, S::min_blocks, MODE, WK, F>;
+  // (passes that generate their rows load none)
+  constexpr bool LOADS = MODE != kSrcInitUniform && MODE != kSrcInitReadMajor && MODE != kSrcInitSplit && MODE != kSrcInitMixed;
+  const bool early = a.n_tiles <= kLookWideTiles;
+  auto kern = k_onesweep<V, S::threads, S::ipt, S::min_blocks, MODE, WK, F, false>;
+  if constexpr (LOADS)
+    if (early) kern = k_onesweep<V, S::threads, S::ipt, S::min_blocks, MODE, WK, F, true>;
   // Attributes are set once per instantiation and device (a bit per device;
   // threads that race here both set the same values).
   // CTAs resident on the whole GPU, per device (set with the attributes, once;
   // threads that race here store the same values).
-  static std::atomic<uint32_t> resident[64];
+  static std::atomic<uint32_t> resident_of[2][64];
+  auto& resident = resident_of[LOADS && early];
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -514,12 +529,12 @@ cudaError_t launch_mode(const PassArgs& a, cudaStream_t st) {
     resident[dev & 63].store(grid_resident, std::memory_order_release);
   }
   PassArgs b = a;
-  b.look_wide = a.n_tiles <= kLookWideTiles ? 1u : 0u;
+  b.look_wide = early ? 1u : 0u;
   b.prefetch = 0;
   if (MODE == kSrcCarried && a.prefetch && (reinterpret_cast<uintptr_t>(a.keys_in) & 15u) == 0 &&
       (reinterpret_cast<uintptr_t>(a.vals_in) & 15u) == 0)
     b.prefetch = grid_resident;
-  return launch_after(b.look_wide != 0, kern, dim3(a.n_tiles), S::threads, smem, st, b);
+  return launch_after(early, kern, dim3(a.n_tiles), S::threads, smem, st, b);
 }
 
 template <class V, class S>
