@@ -825,6 +825,10 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     if (total != pl.N)
       return fail(c, CXBWT_EINVAL, "bucket counts sum to %llu, not the collection's %llu suffixes",
                   (unsigned long long)total, (unsigned long long)pl.N);
+    // (counts that only sum to N past 2^64 would put the part's rows outside B_R)
+    if (part_row0 > pl.N || part_rows > pl.N - part_row0)
+      return fail(c, CXBWT_EINVAL, "the part's rows [%llu, +%llu) by its bucket counts are outside the %llu of the collection",
+                  (unsigned long long)part_row0, (unsigned long long)part_rows, (unsigned long long)pl.N);
     one_slice = part_rows <= m1;
   }
   if (one_slice) {

@@ -60,3 +60,26 @@ def test_empty_part_counts_as_no_slice(flags):
         st = c.stats()
         assert st["builds"] == 1 and st["slices"] == 0 and st["build_ms"] > 0
         assert st["merge_ms"] == 0 and st["merge_launches"] == 0
+
+
+@pytest.mark.parametrize("flags", [0, 1, 64])
+def test_counts_that_wrap_are_rejected(flags):
+    """Counts that sum to N only modulo 2^64 (a part whose rows would start
+    before or end after B_R): EINVAL, by the host, whatever the plan."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    codes, lens = synth.uniform_reads(3000, 12, 3)
+    words, lens = device(binding.pack_codes(codes)), device(lens)
+    N = 3000 * 13
+    with binding.Context(device=0, plan_flags=flags) as c:
+        for first, lo, row0, rows in ((2**64 - 1600, 1, 2**64 - 1600, 1600), (2**64 - 1600, 0, 0, 2**64 - 1600)):
+            counts = np.zeros(binding.BUCKETS, dtype=np.uint64)
+            counts[0], counts[1], counts[2] = first, 1600, N
+            out = torch.zeros(N, dtype=torch.int32, device="cuda")
+            with pytest.raises((binding.CxbwtError, ValueError)) as e:
+                c.build_part(words, lens, lo, lo + 1, row0, rows, out, bucket_counts=counts)
+            assert isinstance(e.value, ValueError) or e.value.status == -1
+        assert c.stats()["builds"] == 0
+        ok = c.bucket_counts(words, lens)
+        c.build_part(words, lens, 0, binding.BUCKETS, 0, N, bucket_counts=ok)
