@@ -1034,6 +1034,15 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   if (merged) {
     if (part) CX_CUDA(c, cudaMemsetAsync(r.d_counts, 0, 5 * 8, st));
     if (c->opt.timing) CX_CUDA(c, cudaEventRecord(c->ev[0], st));
+    if (part && part->given_counts) {
+      // The sort of a part lists its buckets' suffixes and so meets counts of
+      // other reads; the merge plan takes rows of B_R and would not.
+      const uint32_t key_lo = uint32_t(uint64_t(part->lo) << (32 - kBucketBits));
+      const uint32_t key_last = uint32_t((uint64_t(part->hi) << (32 - kBucketBits)) - 1 - key_lo);
+      CX_CUDA(c, launch_expect_rows(r.R, uint32_t(n), key_lo, key_last, part_rows,
+                                    reinterpret_cast<unsigned long long*>(misc + kMiscTotal), r.d_err, c->sm_count, st));
+      r.launches += 2;
+    }
     CX_TRY(merge_run(c, r, part_row0, part_row0 + part_rows, word0, bwt_words, part != nullptr));
     if (!bwt_dev && bwt_words) {
       CX_CUDA(c, cudaMemcpyAsync(out_bwt, r.d_bwt, bwt_words * 4, cudaMemcpyDeviceToHost, st));

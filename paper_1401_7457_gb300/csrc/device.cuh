@@ -31,6 +31,7 @@ constexpr int kRadix = 1 << kRadixBits;
 // Device error word bits.
 constexpr uint32_t kErrTimeout = 1u;
 constexpr uint32_t kErrBounds = 2u;
+constexpr uint32_t kErrCounts = 4u;  // a range holds other than the suffixes its caller counted
 
 struct ReadIndex {
   const uint32_t* words;  // packed store

@@ -150,6 +150,7 @@ constexpr size_t kMiscErr = 4;           // uint32
 constexpr size_t kMiscCounts = 64;       // 5 x uint64
 constexpr size_t kMiscLenStats = 128;    // 4 x uint64
 constexpr size_t kMiscSeg = 192;         // 8 x uint32: group-finish list lengths and work counters
+constexpr size_t kMiscTotal = 224;       // uint64: suffixes of a part's buckets
 constexpr size_t kMiscBytes = 256;
 
 inline uint32_t bits_for(uint32_t x) {  // smallest s with 2^s > x
@@ -290,6 +291,8 @@ inline int take_device_error(cxbwt_ctx* c) {
   if (derr & kErrTimeout) return fail(c, CXBWT_ETIMEOUT, "a radix look-back wait exceeded its limit");
   if (derr & kErrBounds)
     return fail(c, CXBWT_EINTERNAL, "a sort pass or the emission met an out-of-range row or suffix id");
+  if (derr & kErrCounts)
+    return fail(c, CXBWT_EINTERNAL, "the part's buckets do not hold the suffixes that the bucket counts given say");
   return fail(c, CXBWT_EINTERNAL, "device check failed (error word 0x%x)", derr);
 }
 

@@ -309,9 +309,12 @@ __global__ void __launch_bounds__(THREADS) k_list(const ListArgs a) {
 // count of a range, k_pass_hist, adds to six shared counters per suffix kept:
 // for a quarter of 101M suffixes 331 us; so, with
 // the count of the kept keys' digits, about 120: the part 2.29 -> 2.08 ms.)
+// TOTAL: their number alone, for reads of any length that a tile holds (to hold
+// the counts a caller gives against the reads: 82 us for 101M suffixes).
+template <bool TOTAL>
 __global__ void __launch_bounds__(256) k_list_lengths(const ReadIndex R, uint32_t n_reads, uint32_t reads_per_tile,
                                                       uint32_t n_tiles, uint32_t key_lo, uint32_t key_last,
-                                                      uint32_t* __restrict__ hist) {
+                                                      uint32_t* __restrict__ hist, unsigned long long* total) {
   __shared__ uint32_t s_words[kListWords];
   const uint32_t L = R.uniform_len, L1 = L + 1u;
   const bool halves = L1 <= 128u;  // as in k_list
@@ -334,9 +337,27 @@ __global__ void __launch_bounds__(256) k_list_lengths(const ReadIndex R, uint32_
       for (uint32_t i = ra; i < rb; ++i, q += L)
         cnt += window_staged(s_words, q, keep, false, nullptr) - key_lo <= key_last ? 1u : 0u;
     }
+    if (TOTAL) {
+      for (uint32_t kk = k + 256u; kk <= L; kk += 256u) {  // (reads of 256 bases and more: not in halves)
+        const uint32_t left = L - kk;
+        const uint32_t keep_k = left >= 16u ? 0xFFFFFFFFu : ~(0xFFFFFFFFu >> (2u * left));
+        uint32_t q = uint32_t(uint64_t(i0) * L - (w_lo << 4)) + (kk < L ? kk : 0u);
+        for (uint32_t i = i0; i < i1; ++i, q += L)
+          cnt += window_staged(s_words, q, keep_k, false, nullptr) - key_lo <= key_last ? 1u : 0u;
+      }
+    }
     __syncthreads();
   }
-  if (k <= L && cnt) atomicAdd(hist + (L - k), cnt);
+  if (TOTAL) {
+    const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, cnt);
+    if ((threadIdx.x & 31u) == 0 && sum) atomicAdd(total, (unsigned long long)sum);
+  } else if (k <= L && cnt) {
+    atomicAdd(hist + (L - k), cnt);
+  }
+}
+
+__global__ void k_expect_total(const unsigned long long* total, unsigned long long rows, uint32_t* err) {
+  if (*total != rows) atomicOr(err, kErrCounts);
 }
 
 template <class V, int THREADS, int NS>
@@ -389,7 +410,23 @@ cudaError_t launch_list_lengths(const ReadIndex& R, uint32_t n_reads, uint32_t k
   const uint32_t rpt = list_reads_per_tile(R.uniform_len);
   if (R.uniform_len + 1 > uint32_t(kSlots) || !words_fit(rpt, R.uniform_len)) return cudaErrorInvalidValue;
   const uint32_t n_tiles = (n_reads + rpt - 1) / rpt;
-  k_list_lengths<<<std::min(n_tiles, uint32_t(sm_count) * 8), 256, 0, st>>>(R, n_reads, rpt, n_tiles, key_lo, key_last, hist);
+  k_list_lengths<false><<<std::min(n_tiles, uint32_t(sm_count) * 8), 256, 0, st>>>(R, n_reads, rpt, n_tiles, key_lo, key_last,
+                                                                                   hist, nullptr);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_expect_rows(const ReadIndex& R, uint32_t n_reads, uint32_t key_lo, uint32_t key_last, uint64_t rows,
+                               unsigned long long* total, uint32_t* err, int sm_count, cudaStream_t st) {
+  const uint32_t rpt = list_reads_per_tile(R.uniform_len);
+  if (n_reads == 0 || !words_fit(rpt, R.uniform_len)) return cudaErrorInvalidValue;
+  cudaError_t e = cudaMemsetAsync(total, 0, sizeof *total, st);
+  if (e != cudaSuccess) return e;
+  const uint32_t n_tiles = (n_reads + rpt - 1) / rpt;
+  k_list_lengths<true><<<std::min(n_tiles, uint32_t(sm_count) * 8), 256, 0, st>>>(R, n_reads, rpt, n_tiles, key_lo, key_last,
+                                                                                  nullptr, total);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_expect_total<<<1, 1, 0, st>>>(total, rows, err);
   return cudaGetLastError();
 }
 

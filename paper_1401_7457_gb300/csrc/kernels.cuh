@@ -109,6 +109,10 @@ cudaError_t launch_list(const ListArgs& a, int id_bytes, cudaStream_t st);
 // window w has w - key_lo <= key_last: added to hist[0 .. L].
 cudaError_t launch_list_lengths(const ReadIndex& R, uint32_t n_reads, uint32_t key_lo, uint32_t key_last, uint32_t* hist,
                                 int sm_count, cudaStream_t st);
+// Counts the suffixes of that range (reads of one length of at most 4096 bases)
+// into *total; kErrCounts in *err unless there are `rows`.
+cudaError_t launch_expect_rows(const ReadIndex& R, uint32_t n_reads, uint32_t key_lo, uint32_t key_last, uint64_t rows,
+                               unsigned long long* total, uint32_t* err, int sm_count, cudaStream_t st);
 // hist[256 * r ..] becomes its exclusive prefix sums, for r < rows.
 cudaError_t launch_scan_rows(uint32_t* hist, uint32_t rows, cudaStream_t st);
 

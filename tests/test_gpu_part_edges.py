@@ -83,3 +83,29 @@ def test_counts_that_wrap_are_rejected(flags):
         assert c.stats()["builds"] == 0
         ok = c.bucket_counts(words, lens)
         c.build_part(words, lens, 0, binding.BUCKETS, 0, N, bucket_counts=ok)
+
+
+@pytest.mark.parametrize("length,flags", [(12, 64), (100, 64), (127, 64), (128, 65), (255, 64), (256, 64), (300, 64), (528, 64)])
+def test_counts_of_other_reads_are_noticed_by_the_merge_plan(length, flags):
+    """Counts of other reads with the same sum, over a range that holds more or
+    fewer suffixes than they say: an error, as when the part is sorted; the
+    right counts of the same ranges are taken."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    n = 3000 * 100 // (length + 1) + 31
+    a, la = synth.uniform_reads(n, length, 1)
+    b, _ = synth.uniform_reads(n, length, 2)
+    lens, a, b = device(la), device(binding.pack_codes(a)), device(binding.pack_codes(b))
+    with binding.Context(device=0, plan_flags=flags) as c:
+        of_a, of_b = c.bucket_counts(a, lens), c.bucket_counts(b, lens)
+        diff = np.cumsum(of_a.astype(np.int64) - of_b.astype(np.int64))
+        for hi in (int(np.argmax(diff[:-1])) + 1, int(np.argmin(diff[:-1])) + 1):
+            assert diff[hi - 1] != 0
+            for lo, h in ((0, hi), (hi, binding.BUCKETS)):
+                before = c.stats()["merge_launches"]
+                with pytest.raises(binding.CxbwtError) as e:
+                    c.build_part(a, lens, lo, h, int(of_b[:lo].sum()), int(of_b[lo:h].sum()), bucket_counts=of_b)
+                assert e.value.status == -7
+                c.build_part(a, lens, lo, h, int(of_a[:lo].sum()), int(of_a[lo:h].sum()), bucket_counts=of_a)
+                assert c.stats()["merge_launches"] > before
