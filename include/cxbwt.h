@@ -132,12 +132,14 @@ typedef struct {
 /* Sort plans.  Every plan computes the same B_R; they differ in speed only.
  *  AUTO     - for reads of one length in a build of one slice, when the
  *             suffix list is not asked for and tile_items, prefix_len and
- *             plan_flags are 0, the merge plan where it is the faster one (from
- *             about 150,000 reads of 100 bases on): B_R built one suffix length
- *             at a time, each step inserting the symbols before the suffixes
- *             of that length, with no sort of the suffixes (the scheme of
- *             Bauer, Cox & Rosone 2013).  Else GROUPS when the reads are at
- *             most 528 bases, else LSD.
+ *             plan_flags are 0, the merge plan where it is the faster one
+ *             whatever the reads are (alone: from 2^18 reads of 32 to 104 bases
+ *             on, 1.5 and 3 times as many up to 160 and 528; where builds run
+ *             at once, in a batch or a server, with fewer): B_R built one
+ *             suffix length at a time, each step inserting the symbols before
+ *             the suffixes of that length, with no sort of the suffixes (the
+ *             scheme of Bauer, Cox & Rosone 2013).  Parts take it too.  Else
+ *             GROUPS when the reads are at most 528 bases, else LSD.
  *  LSD      - stable LSD radix passes over every 4-base digit of the
  *             A-padded suffixes (Section 3.2 as stated: one pass per digit).
  *  GROUPS   - LSD passes over the first l = 16 (or prefix_len = 12)

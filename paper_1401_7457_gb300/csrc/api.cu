@@ -584,26 +584,60 @@ static int finish_build(cxbwt_ctx* c, Run& r, const Outs& o, uint64_t h2d, size_
   return CXBWT_OK;
 }
 
-// Whether the merge plan (merge.cu) is the faster one for a build, or a part
-// of `rows` of its rows, that a sort would make in one slice.  Fitted to both
-// plans' times with the store in L2 (reads x bases: merge against group plan):
-// 10k x 100 0.56 / 0.21 ms, 100k x 100 0.82 / 0.67, 300k x 100 1.26 / 1.63,
-// 1M x 36 0.84 / 1.62, 1M x 100 2.61 / 4.81, 250k x 400 8.00 / 8.25.  A merge
-// step costs 5.5 us and 11 + 0.115 L ps per read; the group plan 130 us and
-// 36 + 0.113 L ps per suffix, the LSD plan 6 ps per suffix and digit; a part
-// lists its rows among all suffixes (13 ps each by a digit pass, less by the
+// Reads of `len` bases (at most 528) from which on a build takes the merge plan
+// (merge.cu): as many as make it the faster one for unrelated reads, whose sort
+// is the cheapest there is (no groups to finish); reads of a genome at 20x reach
+// that point with fewer.  A build alone, merge / group plan, in ms, unrelated reads
+// and a 20x genome, with the store in L2:
+//   len   reads     unrelated     20x          reads     unrelated     20x
+//   4     5M        0.53 / 0.45   0.53 / 0.44  20M       1.75 / 1.63   1.74 / 1.63
+//   8     2M        0.48 / 0.44   0.48 / 0.44  5M        0.84 / 0.91   0.84 / 0.91
+//   12    500k      0.34 / 0.30   0.33 / 0.30  1M        0.44 / 0.45   0.44 / 0.45
+//   20    300k      0.39 / 0.37   0.40 / 0.37  400k      0.40 / 0.49   0.40 / 0.51
+//   36    200k      0.44 / 0.41   0.45 / 0.41  262k      0.49 / 0.53   0.49 / 0.58
+//   100   200k      0.98 / 0.89   0.99 / 1.15  262k      1.10 / 1.12   1.11 / 1.44
+//   150   250k      1.72 / 1.60   1.72 / 2.18  400k      2.28 / 2.48   2.29 / 3.37
+//   250   400k      5.10 / 4.37   5.12 / 6.39  1M        9.99 / 12.0   9.99 / 16.3
+//   400   250k      7.67 / 5.00   7.69 / 8.18  700k      16.2 / 16.1   16.3 / 23.8
+// Builds that run at once (the workers of a batch or a server) fill one another's
+// gaps, of which the merge plan has more, a launch per suffix length: it is then
+// the faster one with fewer reads.  Time per build, merge / sort, 12 collections
+// of unrelated reads: three at once 16 x 150k 0.12 / 0.13, 100 x 75k 0.32 / 0.31,
+// 100 x 100k 0.35 / 0.40, 250 x 150k 1.28 / 1.41, 300 x 250k 2.91 / 3.00,
+// 400 x 150k 2.91 / 2.41; two at once 16 x 200k 0.17 / 0.17, 100 x 150k 0.53 /
+// 0.58, 250 x 150k 1.46 / 1.44, 250 x 200k 1.78 / 1.91, 300 x 250k 2.98 / 2.97.
+static uint64_t merge_from(uint32_t len, int peers) {
+  if (peers > 1 && len >= 10 && len <= 320) {
+    if (len < 16) return uint64_t(3) << 18;
+    if (len > 255) return uint64_t(1) << 18;
+    return peers > 2 ? uint64_t(1) << 17 : uint64_t(3) << 16;
+  }
+  if (len < 6) return ~uint64_t(0);
+  if (len < 10) return uint64_t(1) << 22;
+  if (len < 16) return uint64_t(1) << 20;
+  if (len < 32) return uint64_t(3) << 17;
+  if (len <= 104) return uint64_t(1) << 18;
+  if (len <= 160) return uint64_t(3) << 17;
+  return uint64_t(3) << 18;
+}
+
+// Whether the merge plan is taken for a build, or a part of `rows` of its rows,
+// that a sort would make in one slice.  Longer reads than the group plan takes:
+// a merge step costs 5.5 us and 11 + 0.115 L ps per read, the LSD plan 6 ps per
+// suffix and digit (600 bases: 1,000 reads 2.5 / 2.2 ms, 10,000 3.3 / 9.1).  A
+// part lists its rows among all suffixes (13 ps each by a digit pass, less by the
 // listing kernel: a quarter of 1M x 100 bases is sorted in 1.91 ms, 2.23 by the
 // formula, and merged in 2.5) and sorts them.
 static bool merge_pays(const cxbwt_ctx* c, const Plan& pl, bool part, uint64_t rows) {
   if (c->opt.algorithm != CXBWT_ALGO_AUTO || c->opt.tile_items || c->opt.prefix_len) return false;
   if (c->opt.plan_flags & CXBWT_PLAN_MERGE) return (c->opt.plan_flags & ~(CXBWT_PLAN_MERGE | CXBWT_PLAN_ID64)) == 0;
   if (c->opt.plan_flags) return false;
+  if (pl.groups && !part) return pl.n >= merge_from(pl.Lmax, c->peers);
   const double L = pl.Lmax, n = double(pl.n);
   const double merge_us = (L + 1) * (5.5 + n * (11.0 + 0.115 * L) * 1e-6);
   double sort_us = 130.0;
   if (!pl.groups) sort_us += double(pl.N) * ((L + 3) / 4) * 6.0e-6;
-  else if (part) sort_us += double(pl.N) * 13.0e-6 + double(rows) * (20.0 + 0.113 * L) * 1e-6;
-  else sort_us += double(pl.N) * (36.0 + 0.113 * L) * 1e-6;
+  else sort_us += double(pl.N) * 13.0e-6 + double(rows) * (20.0 + 0.113 * L) * 1e-6;
   return merge_us < sort_us;
 }
 

@@ -58,6 +58,7 @@ struct cxbwt_ctx {
   // Autotuner choices (autotune.cu), one per maximum read length and size
   // class.  Used when the options leave tile, algorithm and depth automatic.
   std::vector<cxbwt::host::TunedPlan> tuned;
+  int peers = 1;                          // builds that run at once with this context's, its own counted
   void* batch_pool = nullptr;             // worker contexts of cxbwt_build_batch (batch.cu), created on first use
   void (*batch_pool_free)(void*) = nullptr;
 };

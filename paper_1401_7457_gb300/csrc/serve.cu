@@ -63,6 +63,7 @@ struct cxbwt_server {
   uint64_t next_ticket = 1;
   uint64_t pack_cap = 0;
   bool stop = false;
+  size_t running = 0;  // workers that build now
   uint64_t completed = 0, packs = 0, bases = 0;
 };
 
@@ -99,6 +100,8 @@ void worker_loop(cxbwt_server* s, int w) {
       }
       const auto now = Clock::now();
       for (Req* q : take) q->t_start = now;
+      ++s->running;
+      ctx->peers = int(std::min(s->ctxs.size(), s->running + s->queue.size()));
     }
     colls.clear();
     for (Req* q : take) {
@@ -129,6 +132,7 @@ void worker_loop(cxbwt_server* s, int w) {
       }
       s->completed += take.size();
       s->packs += 1;
+      --s->running;
     }
     s->cv_done.notify_all();
   }

@@ -1,0 +1,33 @@
+"""Which builds take the merge plan by themselves: on either side of the rule's
+lines, every result the group plan's."""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def reads(n, length):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n + length)
+    words = torch.randint(-2**31, 2**31, ((n * length + 15) // 16,), generator=g, device="cuda").to(torch.int32)
+    if n * length % 16:  # the bits after the last base
+        words[-1] &= -1 << (32 - 2 * (n * length % 16))
+    return words, torch.full((n,), length, dtype=torch.int32, device="cuda")
+
+
+@pytest.mark.parametrize("n,length,merged", [
+    (100_000, 1, False), (1_000_000, 4, False), (1_000_000, 8, False), (4_194_304, 8, True), (50_000, 12, False),
+    (1_048_576, 12, True), (100_000, 20, False), (393_215, 20, False), (393_216, 20, True), (150_000, 36, False),
+    (262_143, 50, False), (262_144, 50, True), (200_000, 100, False), (262_144, 105, False), (250_000, 150, False),
+    (393_216, 150, True), (250_000, 250, False), (250_000, 400, False), (786_432, 200, True)])
+def test_merge_plan_by_reads_and_bases(n, length, merged):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    words, lens = reads(n, length)
+    with binding.Context(device=0) as c, binding.Context(device=0, algorithm=binding.Context.ALGO_GROUPS) as sort:
+        got, want = c.build(words, lens), sort.build(words, lens)
+        assert (c.stats()["merge_launches"] > 0) == merged
+        assert sort.stats()["merge_launches"] == 0
+    for a, b in zip(got[:3], want[:3]):
+        assert torch.equal(a, b)
