@@ -488,6 +488,7 @@ extern "C" int cxbwt_build_batch(cxbwt_ctx* c, const cxbwt_collection* colls, ui
     c->stats.h2d_bytes += wc->stats.h2d_bytes;
     c->stats.d2h_bytes += wc->stats.d2h_bytes;
     c->stats.slices += wc->stats.slices;
+    c->stats.merge_launches += wc->stats.merge_launches;
     wc->stats = cxbwt_stats{};
   }
   return status;

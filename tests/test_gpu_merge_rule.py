@@ -15,6 +15,30 @@ def reads(n, length):
     return words, torch.full((n,), length, dtype=torch.int32, device="cuda")
 
 
+@pytest.mark.parametrize("n,length,workers,k,merged", [
+    (140_000, 50, 3, 3, True), (120_000, 50, 3, 3, False), (140_000, 50, 2, 3, False), (200_000, 50, 2, 3, True),
+    (140_000, 50, 3, 1, False), (800_000, 12, 3, 3, True), (150_000, 15, 3, 3, False), (140_000, 330, 3, 3, False)])
+def test_merge_plan_in_batches(n, length, workers, k, merged):
+    """Builds that run at once take it from fewer reads on; the batch's counters
+    include its steps."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    words, lens = reads(n, length)
+    N = n * (length + 1)
+    outs = [(torch.zeros((N + 15) // 16, dtype=torch.int32, device="cuda"), torch.zeros(n, dtype=torch.int64, device="cuda"),
+             torch.zeros(5, dtype=torch.int64, device="cuda")) for _ in range(k)]
+    with binding.Context(device=0, batch_workers=workers) as c, \
+            binding.Context(device=0, algorithm=binding.Context.ALGO_GROUPS) as sort:
+        want = sort.build(words, lens)
+        c.build_batch([(words, lens, *o) for o in outs])
+        torch.cuda.synchronize()
+        assert c.stats()["builds"] == k and c.stats()["merge_launches"] == (k * (length + 1) if merged else 0)
+    for o in outs:
+        for a, b in zip(o, want[:3]):
+            assert torch.equal(a, b)
+
+
 @pytest.mark.parametrize("n,length,merged", [
     (100_000, 1, False), (1_000_000, 4, False), (1_000_000, 8, False), (4_194_304, 8, True), (50_000, 12, False),
     (1_048_576, 12, True), (100_000, 20, False), (393_215, 20, False), (393_216, 20, True), (150_000, 36, False),
