@@ -303,9 +303,12 @@ inline void* vptr(void* base, int idb, uint64_t row) { return static_cast<char*>
 // another: each 4 bases less is a digit pass less, and pays while few suffixes
 // share their first l bases by chance (at most N / 4^l = 4 rows with 8 bases,
 // half a row with 12: 154k suffixes 141 us with l = 16, 119 with 8; 1.01M 170
-// and 160 with 12).
+// and 160 with 12).  Reads of at most 16 bases have no groups with l = 16, and
+// l = 12 spares a pass but adds the finish: up to 2^20 suffixes (16 bases: 1.02M 155
+// and 142 us; 5.1M 288 and 316; 13 bases: 1.4M 155 and 172).
 inline uint32_t auto_depth(uint64_t n_suffixes, uint32_t max_len) {
-  const uint32_t d = n_suffixes <= (uint64_t(1) << 18) ? 8u : n_suffixes <= (uint64_t(1) << 23) ? 12u : 16u;
+  const uint64_t deep = uint64_t(1) << (max_len <= 16 ? 20 : 23);
+  const uint32_t d = n_suffixes <= (uint64_t(1) << 18) ? 8u : n_suffixes <= deep ? 12u : 16u;
   // (no wider keys for it than 16 words, whose group sorts hold fewer rows)
   return max_len > d && segsort_words(max_len, d) && segsort_words(max_len, d) <= 16 ? d : 16u;
 }
