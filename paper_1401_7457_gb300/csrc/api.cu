@@ -622,23 +622,29 @@ static uint64_t merge_from(uint32_t len, int peers) {
 }
 
 // Whether the merge plan is taken for a build, or a part of `rows` of its rows,
-// that a sort would make in one slice.  Longer reads than the group plan takes:
-// a merge step costs 5.5 us and 11 + 0.115 L ps per read, the LSD plan 6 ps per
-// suffix and digit (600 bases: 1,000 reads 2.5 / 2.2 ms, 10,000 3.3 / 9.1).  A
-// part lists its rows among all suffixes (13 ps each by a digit pass, less by the
-// listing kernel: a quarter of 1M x 100 bases is sorted in 1.91 ms, 2.23 by the
-// formula, and merged in 2.5) and sorts them.
+// that a sort would make in one slice.  A part's merge costs as much as the whole
+// build's, its sort the listing of all suffixes and the sort of its own: the
+// merge plan is taken for parts of nearly all rows, and of fewer the more reads
+// there are past the line for whole builds (merge / sort, in ms, unrelated reads:
+// 262k x 50 bases, all rows 0.69 / 0.85, half 0.69 / 0.56; 600k x 100, all 1.90 /
+// 2.70, half 1.87 / 1.65; 1.1M x 100, half 2.91 / 2.84; 2M x 100, half 4.34 /
+// 5.04, a third 4.29 / 3.73; 4M x 100, half 7.83 / 9.92).
+// Longer reads than the group plan takes: a merge step costs 5.5 us and 11 +
+// 0.115 L ps per read, the LSD plan 6 ps per suffix and digit (600 bases: 1,000
+// reads 2.5 / 2.2 ms, 10,000 3.3 / 9.1).
 static bool merge_pays(const cxbwt_ctx* c, const Plan& pl, bool part, uint64_t rows) {
   if (c->opt.algorithm != CXBWT_ALGO_AUTO || c->opt.tile_items || c->opt.prefix_len) return false;
   if (c->opt.plan_flags & CXBWT_PLAN_MERGE) return (c->opt.plan_flags & ~(CXBWT_PLAN_MERGE | CXBWT_PLAN_ID64)) == 0;
   if (c->opt.plan_flags) return false;
-  if (pl.groups && !part) return pl.n >= merge_from(pl.Lmax, c->peers);
+  if (pl.groups) {
+    const uint64_t from = merge_from(pl.Lmax, part ? 1 : c->peers);
+    if (pl.n < from) return false;
+    const uint64_t left_out = pl.N - (part ? rows : pl.N);  // rows of other parts
+    return left_out <= (pl.n / 6 >= from ? pl.N / 2 : pl.n / 2 >= from ? pl.N / 4 : pl.N / 16);
+  }
   const double L = pl.Lmax, n = double(pl.n);
   const double merge_us = (L + 1) * (5.5 + n * (11.0 + 0.115 * L) * 1e-6);
-  double sort_us = 130.0;
-  if (!pl.groups) sort_us += double(pl.N) * ((L + 3) / 4) * 6.0e-6;
-  else sort_us += double(pl.N) * 13.0e-6 + double(rows) * (20.0 + 0.113 * L) * 1e-6;
-  return merge_us < sort_us;
+  return merge_us < 130.0 + double(pl.N) * ((L + 3) / 4) * 6.0e-6;
 }
 
 int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* lens, uint32_t* out_bwt,

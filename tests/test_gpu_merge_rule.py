@@ -55,3 +55,30 @@ def test_merge_plan_by_reads_and_bases(n, length, merged):
         assert sort.stats()["merge_launches"] == 0
     for a, b in zip(got[:3], want[:3]):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n,length,share,merged", [
+    (100_000, 8, 0.5, False), (10_000, 12, 0.9, False), (262_144, 40, 0.5, False), (262_144, 40, 0.97, True),
+    (524_288, 40, 0.6, False), (524_288, 40, 0.9, True), (1_572_864, 40, 0.4, False), (1_572_864, 40, 0.6, True)])
+def test_merge_plan_for_parts(n, length, share, merged):
+    """Parts of a share of the rows; with the rest, the whole of the group plan's."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    words, lens = reads(n, length)
+    N = n * (length + 1)
+    with binding.Context(device=0) as c, binding.Context(device=0, algorithm=binding.Context.ALGO_GROUPS) as sort:
+        counts = c.bucket_counts(words, lens)
+        before = counts.cumsum()
+        hi = int((before <= share * N).sum())
+        rows = int(before[hi - 1])
+        got = torch.zeros((N + 15) // 16 + 1, dtype=torch.int32, device="cuda")
+        w, dollar, cnt = c.build_part(words, lens, 0, hi, 0, rows, bucket_counts=counts)
+        assert (c.stats()["merge_launches"] > 0) == merged
+        got[:w.numel()] |= w
+        w, d, k = sort.build_part(words, lens, hi, binding.BUCKETS, rows, N - rows, bucket_counts=counts)
+        got[rows // 16:rows // 16 + w.numel()] |= w
+        want = sort.build(words, lens)
+    assert torch.equal(got[:(N + 15) // 16], want[0])
+    none = torch.full_like(d, -1)
+    assert torch.equal(torch.where(dollar == none, d, dollar), want[1]) and torch.equal(cnt + k, want[2])
