@@ -476,7 +476,7 @@ def run_batch_bench(args, rank, world):
     chosen = {}
     for (L, cls), t in sorted(picks.items()):
         plan = f"groups l={t['prefix_len']}" if t['algorithm'] == 2 else "lsd"
-        k = f"tile {t['tile_items']}, {plan}"
+        k = "merge" if t['algorithm'] == 3 else f"tile {t['tile_items']}, {plan}"
         chosen[k] = chosen.get(k, 0) + 1
     line = {"metric": METRIC, "value": bases / out["batched"] / 1e9, "unit": UNIT, "n_gpus": 1, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": out["batched"] * 1e3, "higher_is_better": True, "scaling": "weak",

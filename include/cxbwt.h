@@ -148,6 +148,8 @@ typedef struct {
 #define CXBWT_ALGO_AUTO 0
 #define CXBWT_ALGO_LSD 1
 #define CXBWT_ALGO_GROUPS 2
+/* The merge plan, as cxbwt_autotune names it; not an option (see AUTO). */
+#define CXBWT_ALGO_MERGE 3
 
 /* Counters accumulated by a context since creation or cxbwt_reset_stats. */
 typedef struct {
@@ -363,19 +365,22 @@ int cxbwt_server_counters(cxbwt_server* s, uint64_t* completed, uint64_t* packs,
  * Times every candidate plan on one collection (device or host buffers) and
  * keeps the fastest in the context for builds of the same maximum read
  * length and size class (N within a factor of two) whose options leave
- * tile_items, algorithm and prefix_len automatic.  Candidates: tiles of
- * 4096 or 8192 items (2048, 3072 or 4096 when the build carries 64-bit
- * suffix ids) x the group plan with l = 16 (reads of at most 528 bases) or
- * l = 12 (at most 524), or the LSD plan.  The radix digit is 8 bits (the
+ * tile_items, algorithm and prefix_len automatic.  Candidates: the merge
+ * plan for reads of one length (plan_flags 0); tiles of 4096 or 8192 items
+ * (1024 too up to 2^19 suffixes; 2048, 3072 or 4096 when the build carries
+ * 64-bit suffix ids) x the group plan with l = 16 (reads of at most 528 bases),
+ * l = 12 (at most 524) or l = 8 (up to 2^18 suffixes), or the LSD plan.  A
+ * choice of the merge plan leaves builds with the suffix list, slices and parts
+ * to the automatic rule.  The radix digit is 8 bits (the
  * only width built).  scratch_bwt (ceil(N / 16) words) and
  * scratch_dollar_pos (n_reads, may be NULL) receive the BWT; every candidate
  * produces the same one. */
 typedef struct {
   int tile_items;
-  int algorithm;   /* CXBWT_ALGO_GROUPS or CXBWT_ALGO_LSD */
+  int algorithm;   /* CXBWT_ALGO_GROUPS, CXBWT_ALGO_LSD or CXBWT_ALGO_MERGE (tile_items 0 then) */
   int digit_bits;
   float best_ms;   /* device time of one build with the chosen plan */
-  int prefix_len;  /* l of the chosen group plan (12 or 16); 0 for the LSD plan */
+  int prefix_len;  /* l of the chosen group plan (8, 12 or 16); 0 for the others */
 } cxbwt_tuning;
 int cxbwt_autotune(cxbwt_ctx* ctx, const uint32_t* reads_2bit, uint64_t n_reads, const uint32_t* lens,
                    uint32_t* scratch_bwt, uint64_t* scratch_dollar_pos, void* stream, cxbwt_tuning* out);

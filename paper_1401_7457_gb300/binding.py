@@ -335,6 +335,7 @@ class Context:
     """One cxbwt context (device workspace + bookkeeping) on one device."""
 
     ALGO_AUTO, ALGO_LSD, ALGO_GROUPS = 0, 1, 2
+    ALGO_MERGE = 3  # named by autotune, not an option
     PLAN_ID64, PLAN_READ_MAJOR, PLAN_TEST_STALL, PLAN_CARRY_BASE, PLAN_NO_PREFETCH = 1, 2, 4, 8, 16
     PLAN_DIGIT_LISTING, PLAN_MERGE = 32, 64
 

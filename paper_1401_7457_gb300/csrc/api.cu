@@ -632,11 +632,15 @@ static uint64_t merge_from(uint32_t len, int peers) {
 // Longer reads than the group plan takes: a merge step costs 5.5 us and 11 +
 // 0.115 L ps per read, the LSD plan 6 ps per suffix and digit (600 bases: 1,000
 // reads 2.5 / 2.2 ms, 10,000 3.3 / 9.1).
-static bool merge_pays(const cxbwt_ctx* c, const Plan& pl, bool part, uint64_t rows) {
+// tuned: the autotuner's choice for builds of this class (-1: none; it timed
+// whole builds, alone).
+static bool merge_pays(const cxbwt_ctx* c, const Plan& pl, bool part, uint64_t rows, int tuned) {
   if (c->opt.algorithm != CXBWT_ALGO_AUTO || c->opt.tile_items || c->opt.prefix_len) return false;
   if (c->opt.plan_flags & CXBWT_PLAN_MERGE) return (c->opt.plan_flags & ~(CXBWT_PLAN_MERGE | CXBWT_PLAN_ID64)) == 0;
   if (c->opt.plan_flags) return false;
-  if (pl.groups) {
+  if (tuned >= 0 && !part && c->peers == 1) return tuned == CXBWT_ALGO_MERGE;
+  if (tuned >= 0 && part && tuned != CXBWT_ALGO_MERGE) return false;
+  if (pl.seg_words) {
     const uint64_t from = merge_from(pl.Lmax, part ? 1 : c->peers);
     if (pl.n < from) return false;
     const uint64_t left_out = pl.N - (part ? rows : pl.N);  // rows of other parts
@@ -727,11 +731,13 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   pl.W = (pl.Lmax + 15) / 16;
   pl.len_passes = pl.uniform ? 0 : (pl.Lmax > 255 ? 2 : 1);
   pl.n_words = (sum + 15) / 16;
-  int algorithm = c->opt.algorithm, tile_items = c->opt.tile_items, depth = c->opt.prefix_len;
+  int algorithm = c->opt.algorithm, tile_items = c->opt.tile_items, depth = c->opt.prefix_len, tuned = -1;
   {
     int t_tile = 0, t_algo = 0, t_depth = 0;
     if (tuned_choice(c, pl.Lmax, pl.N, &t_tile, &t_algo, &t_depth)) {
-      if (algorithm == CXBWT_ALGO_AUTO) algorithm = t_algo;
+      tuned = t_algo;
+      // (what the merge plan does not build is sorted by the automatic plan)
+      if (algorithm == CXBWT_ALGO_AUTO && t_algo != CXBWT_ALGO_MERGE) algorithm = t_algo;
       if (tile_items == 0) tile_items = t_tile;
       if (depth == 0) depth = t_depth;
     }
@@ -847,11 +853,15 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   std::vector<uint32_t> P_host;  // per-position 4-mer counts, when the slices were planned from them
   bool refined = false;          // an 8-base bucket was split into 16-base ones
   // The merge plan sorts no slices.
-  bool merged = !out_sa && !part && merge_pays(c, pl, false, pl.N) &&
+  bool merged = !out_sa && !part && merge_pays(c, pl, false, pl.N, tuned) &&
                 pl.N <= ((c->opt.plan_flags & CXBWT_PLAN_MERGE) ? m1_bytes : m1) && merge_fits(c, pl, out_more);
   // A part whose bucket counts are given and that fits one slice needs no more
   // of them than the sums before, in and after it.
   bool one_slice = false;
+  if (pl.groups && pl.depth < 12 && (part || (pl.N > m1 && !merged))) {
+    pl.depth = 16;  // (8, by the autotuner's choice, is for builds of one slice)
+    pl.seg_words = segsort_words(pl.Lmax, pl.depth);
+  }
   if (part && part->given_counts && !counts_only && pl.groups) {
     const uint64_t* bc = part->given_counts;
     auto sum = [&](size_t lo, size_t hi) {
@@ -1070,7 +1080,7 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
     return finish_build(c, r, Outs{out_bwt, out_dollar, out_counts, out_sa, bwt_dev, dollar_dev, counts_dev, sa_dev}, h2d,
                         0);
   }
-  if (part && merge_pays(c, pl, true, part_rows) && pl.N <= m1 && merge_fits(c, pl, 0)) merged = true;
+  if (part && merge_pays(c, pl, true, part_rows, tuned) && pl.N <= m1 && merge_fits(c, pl, 0)) merged = true;
   if (merged) {
     if (part) CX_CUDA(c, cudaMemsetAsync(r.d_counts, 0, 5 * 8, st));
     if (c->opt.timing) CX_CUDA(c, cudaEventRecord(c->ev[0], st));

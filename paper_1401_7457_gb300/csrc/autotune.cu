@@ -1,12 +1,13 @@
 // cxbwt_autotune: choose the tile shape, the sort plan and the group plan's
 // depth by timing them.
 //
-// For one collection (device memory), every candidate (tile of 4096 or 8192
-// items with 32-bit suffix ids, of 2048, 3072 or 4096 with 64-bit ones;
-// the group plan with its first l = 16 or l = 12 bases sorted by LSD passes
-// (four or three passes, then groups sharing those bases finished on chip),
-// or the LSD plan, where they apply) is built three times and the last two
-// are timed with CUDA events on the caller's stream; the fastest choice is
+// For one collection (device memory), every candidate (the merge plan for
+// reads of one length; tiles of 4096 or 8192 items with 32-bit suffix ids, and
+// of 1024 in small builds, of 2048, 3072 or 4096 with 64-bit ones; the group
+// plan with its first l = 16 or l = 12 bases, 8 in small builds, sorted by LSD
+// passes, then groups sharing those bases finished on chip, or the LSD plan,
+// where they apply) is built three times, small ones nine times, and all but
+// the first are timed with CUDA events on the caller's stream; the fastest is
 // kept in the context for builds of the same maximum read length and size
 // class (N within a factor of two).  Builds whose options leave the tile,
 // the plan and prefix_len automatic then use it.  Every candidate gives the
@@ -17,6 +18,7 @@
 #include <cuda_runtime.h>
 
 #include "host.cuh"
+#include "merge.cuh"
 
 using namespace cxbwt;
 using namespace cxbwt::host;
@@ -53,8 +55,15 @@ extern "C" int cxbwt_autotune(cxbwt_ctx* c, const uint32_t* reads_2bit, uint64_t
   c->tuned.clear();
   struct Cand { int tile, algo, depth; };
   std::vector<Cand> cands;
-  const std::vector<int> tiles = probe.idb == 8 ? std::vector<int>{2048, 3072, 4096} : std::vector<int>{4096, 8192};
+  // What an untuned context would take is among the candidates: small tiles and
+  // l = 8 where those are its choice, the merge plan wherever it can be built.
+  if (probe.uniform && Lmax <= kMergeMaxLen && saved.algorithm == CXBWT_ALGO_AUTO && !saved.tile_items &&
+      !saved.prefix_len && !(saved.plan_flags & ~CXBWT_PLAN_MERGE))
+    cands.push_back(Cand{0, CXBWT_ALGO_MERGE, 0});
+  std::vector<int> tiles = probe.idb == 8 ? std::vector<int>{2048, 3072, 4096} : std::vector<int>{4096, 8192};
+  if (probe.idb == 4 && N <= kSmallRows) tiles.insert(tiles.begin(), kSmallTile);
   for (int t : tiles) {
+    if (auto_depth(N, Lmax) == 8) cands.push_back(Cand{t, CXBWT_ALGO_GROUPS, 8});
     if (segsort_words(Lmax, 16)) cands.push_back(Cand{t, CXBWT_ALGO_GROUPS, 16});
     if (segsort_words(Lmax, 12) && Lmax > 12) cands.push_back(Cand{t, CXBWT_ALGO_GROUPS, 12});
     cands.push_back(Cand{t, CXBWT_ALGO_LSD, 0});
@@ -65,14 +74,18 @@ extern "C" int cxbwt_autotune(cxbwt_ctx* c, const uint32_t* reads_2bit, uint64_t
   float best = -1.f;
   Cand pick{0, 0, 0};
   int status = CXBWT_OK;
+  const int reps = N <= kSmallRows ? 9 : 3;
   for (const Cand& cd : cands) {
+    const bool merge = cd.algo == CXBWT_ALGO_MERGE;
     c->opt.tile_items = cd.tile;
-    c->opt.algorithm = cd.algo;
+    c->opt.algorithm = merge ? CXBWT_ALGO_AUTO : cd.algo;
     c->opt.prefix_len = cd.depth;
+    c->opt.plan_flags = merge ? saved.plan_flags | CXBWT_PLAN_MERGE : saved.plan_flags;
     c->opt.async = 0;
+    const uint64_t merged_before = c->stats.merge_launches;
     float ms_best = 1e30f;
     int st_c = CXBWT_OK;
-    for (int rep = 0; rep < 3 && st_c == CXBWT_OK; ++rep) {
+    for (int rep = 0; rep < reps && st_c == CXBWT_OK; ++rep) {
       cudaEventRecord(e0, st);
       st_c = build_impl(c, reads_2bit, n_reads, lens, scratch_bwt, scratch_dollar_pos, nullptr, nullptr, stream);
       cudaEventRecord(e1, st);
@@ -85,10 +98,13 @@ extern "C" int cxbwt_autotune(cxbwt_ctx* c, const uint32_t* reads_2bit, uint64_t
       status = st_c;
       break;
     }
+    const bool merged = c->stats.merge_launches > merged_before;
+    if (merge && !merged) continue;  // it does not fit the budget: its builds were sorted
     if (best < 0 || ms_best < best) {
       best = ms_best;
       pick = cd;
     }
+    if (merge && (saved.plan_flags & CXBWT_PLAN_MERGE)) break;  // what this context's builds take anyway
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);

@@ -26,7 +26,8 @@ struct DevBuf {
 constexpr uint64_t kTimeoutNs = 1000000000ull;  // look-back waits give up after 1 s
 
 // An autotuned plan for builds of one maximum read length and size class
-// (key: tune_key): tile items, algorithm, and the group plan's depth l.
+// (key: tune_key): tile items, algorithm (CXBWT_ALGO_MERGE: the merge plan), and
+// the group plan's depth l.
 struct TunedPlan {
   uint64_t key;
   int tile, algo, depth;
