@@ -827,9 +827,10 @@ int build_impl(cxbwt_ctx* c, const uint32_t* reads, uint64_t n, const uint32_t* 
   const uint64_t fixed = uint64_t(pl.Lmax) * kRadix * 4 + uint64_t(pl.D + pl.len_passes + 5) * kRadix * 4 +
                          uint64_t(pl.W) * 4 * kRadix * 4 + (uint64_t(1) << kBucketBits) * 8 + status_bytes + (1u << 20);
   // Buffers sized per slice are reused (or regrown) by this build: they do
-  // not count against what it may take.
+  // not count against what it may take.  Nor do the merge plan's, given back
+  // when others need their bytes (ensure).
   const uint64_t reusable = c->vals[0].cap + c->vals[1].cap + c->keys[0].cap + c->keys[1].cap + c->status.cap +
-                            c->seglist.cap + c->out_sa.cap;
+                            c->seglist.cap + c->out_sa.cap + c->mstatus.cap + c->mtables.cap;
   const uint64_t held_fixed = c->held - reusable;
   // Output staging for host buffers is granted below, after the slices are
   // planned: count what it will add to what is held now (a whole build's size

@@ -92,12 +92,24 @@ inline int fail(cxbwt_ctx* c, int status, const char* fmt, ...) {
     if (s_ != CXBWT_OK) return s_; \
   } while (0)
 
-// Grow-only device buffer within the context's budget.
+inline void release(cxbwt_ctx* c, DevBuf& b) {
+  if (b.p) cudaFree(b.p);
+  c->held -= b.cap;
+  b.p = nullptr;
+  b.cap = 0;
+}
+
+// Grow-only device buffer within the context's budget.  The merge plan's own
+// buffers make room for others (cudaFree waits for what still uses them).
 inline int ensure(cxbwt_ctx* c, DevBuf& b, size_t bytes, const char* what) {
   if (b.cap >= bytes) return CXBWT_OK;
   // Large buffers grow in 2 MB steps (fewer regrows), small ones in 64 KB steps.
   const size_t step = bytes >= (size_t(64) << 20) ? (size_t(1) << 21) : (size_t(1) << 16);
   const size_t want = std::max<size_t>((bytes + step - 1) & ~(step - 1), step);
+  if (c->held - b.cap + want > c->budget && &b != &c->mstatus && &b != &c->mtables) {
+    release(c, c->mstatus);
+    release(c, c->mtables);
+  }
   if (c->held - b.cap + want > c->budget)
     return fail(c, CXBWT_ENOMEM, "device budget of %llu bytes exceeded growing %s to %zu bytes",
                 (unsigned long long)c->budget, what, want);
@@ -117,13 +129,6 @@ inline int ensure(cxbwt_ctx* c, DevBuf& b, size_t bytes, const char* what) {
   b.cap = want;
   c->held += want;
   return CXBWT_OK;
-}
-
-inline void release(cxbwt_ctx* c, DevBuf& b) {
-  if (b.p) cudaFree(b.p);
-  c->held -= b.cap;
-  b.p = nullptr;
-  b.cap = 0;
 }
 
 inline bool is_device_ptr(const void* p) {
