@@ -16,7 +16,8 @@ Extra keys: ``e2e`` (same metric through the C ABI with pinned host buffers,
 input copy and the streamed BWT, $ rows and counts inside the timed region),
 ``roofline`` of the dominant kernel (the onesweep carried-key digit pass:
 key and id read and written, 24 B per item with 64-bit ids, each pass timed
-live between the library's own CUDA events), ``phases`` (every phase of a
+live between the library's own CUDA events; the merge step where the merge
+plan builds the workload), ``phases`` (every phase of a
 build against its own algorithmic bytes), ``cpu_baseline`` (the oracle on a
 bounded sample on this host's cores, rank 0 only), ``clocks`` (sampled during
 the timed region), ``gpu_launches`` and ``config2`` (the same measurement on
@@ -327,6 +328,41 @@ def phase_rates(st, steps, n_reads, bases, idb, peak):
         gbs = nbytes / (ms * 1e-3) / 1e9
         out[name] = {"ms_per_step": ms, "bytes_per_step": nbytes, "gbs": gbs, "frac_of_hbm": gbs / peak}
     return out
+
+
+def roofline_of(st, steps, n_reads, bases, idb, peak, peak_kind):
+    """The dominant kernel of `steps` builds with counters st (timing enabled)
+    against the copy bandwidth `peak`.
+
+    A sorted build's is the onesweep digit pass that loads the key window the
+    previous pass carried: per item the key (4 B) and the id (idb bytes), read
+    and written, each launch timed between its own events on the build stream.
+    A build by the merge plan has no such pass: there it is the merge step, whose
+    algorithmic bytes are those of phase_rates' merge steps and whose time is the
+    build's (tables and first suffixes included) over the steps."""
+    merged = st.get("merge_launches", 0) > 0 and st["carried_pass_launches"] == 0
+    if merged:
+        launches = st["merge_launches"]
+        pass_ms = st["merge_ms"] / launches
+        items = (bases + n_reads) / 2  # rows of a step, on average
+        step_bytes = phase_rates(st, steps, n_reads, bases, idb, peak)["merge_steps"]["bytes_per_step"] * steps / launches
+        per_item, traffic = step_bytes / items, None
+    else:
+        launches = max(st["carried_pass_launches"], 1)
+        pass_ms = st["carried_pass_ms"] / launches
+        items = st["carried_pass_items"] / launches
+        per_item = 2 * (4 + idb)
+        profiled = profiled_traffic(idb)
+        traffic = None if profiled is None else profiled * items
+    achieved = per_item * items / (pass_ms * 1e-3) / 1e9 if pass_ms > 0 else 0.0
+    return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+            "traffic": traffic,
+            "peak_source": f"{peak_kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
+            else "fallback 6.8 TB/s",
+            "kernel": "k_merge_step, one suffix length" if merged else "k_onesweep, carried-key digit pass",
+            "launches_per_step": (launches if merged else st["carried_pass_launches"]) / steps,
+            "bytes_per_item": per_item, "items_per_launch": items, "algorithmic_bytes_per_launch": per_item * items,
+            "avg_launch_ms": pass_ms, "frac_of_nominal_8tbs": achieved / 8000.0}
 
 
 def cpu_model():
@@ -1015,27 +1051,9 @@ def measure(args, dist, world, local, dev, desc, codes, lens, steps, e2e_steps):
     del ctx
     value, total_ms = aggregate(dist, sum(ms), bases, world, steps)
 
-    # Dominant kernel: the onesweep digit pass that loads the key window the
-    # previous pass carried.  Its algorithmic bytes per item are the key
-    # (4 B) and the id (4 or 8 B), read and written; each launch is timed
-    # between its own events on the build stream.
     idb = 8 if args.plan_flags & 1 else id_bytes(n, int(lens.max()), int((bases + 15) // 16) * 4)
-    bytes_per_item = 2 * (4 + idb)
-    launches = max(st["carried_pass_launches"], 1)
-    pass_ms = st["carried_pass_ms"] / launches
-    items_per_launch = st["carried_pass_items"] / launches
-    achieved = bytes_per_item * items_per_launch / (pass_ms * 1e-3) / 1e9 if pass_ms > 0 else 0.0
     peak, peak_kind = peak_hbm()
-    traffic_per_item = profiled_traffic(idb)
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "traffic": None if traffic_per_item is None else traffic_per_item * items_per_launch,
-                "peak_source": f"{peak_kind} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
-                else "fallback 6.8 TB/s",
-                "kernel": "k_onesweep, carried-key digit pass",
-                "launches_per_step": st["carried_pass_launches"] / steps,
-                "bytes_per_item": bytes_per_item, "items_per_launch": items_per_launch,
-                "algorithmic_bytes_per_launch": bytes_per_item * items_per_launch,
-                "avg_launch_ms": pass_ms, "frac_of_nominal_8tbs": achieved / 8000.0}
+    roofline = roofline_of(st, steps, n, bases, idb, peak, peak_kind)
 
     # End to end through the C ABI with pinned host buffers (copies inside the timed region).
     h_words = torch.from_numpy(words.view(np.int32)).pin_memory()
