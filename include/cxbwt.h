@@ -78,13 +78,15 @@ typedef struct {
   int prefix_len;               /* l of the group plan (Section 3.1: suffixes sharing their first l bases
                                    form one partition): its LSD passes sort the first l bases and each
                                    partition is finished on chip.  0 = automatic (the autotuned value for
-                                   the build's size class, else 16), 12 or 16; other values give
-                                   CXBWT_EUNSUPPORTED.  Slices and parts are planned from buckets of 4 or
-                                   8 bases (16 when refined) whatever l is */
+                                   the build's size class, else 8 up to 2^18 suffixes, 12 up to 2^23 (2^20
+                                   for reads of at most 16 bases) and 16 above, and in slices and parts),
+                                   12 or 16; other values give CXBWT_EUNSUPPORTED.  Slices and parts are
+                                   planned from buckets of 4 or 8 bases (16 when refined) whatever l is */
   int digit_bits;               /* radix digit width; 8 is the only width built (0 = 8, others give
                                    CXBWT_EUNSUPPORTED) */
-  int tile_items;               /* items per radix tile: 0 = automatic (4096); 4096 or 8192 with 32-bit
-                                   suffix ids, 2048, 3072 or 4096 with 64-bit ones */
+  int tile_items;               /* items per radix tile: 0 = automatic (1024 up to 2^19 suffixes with 32-bit
+                                   ids, else 4096); 4096 or 8192 with 32-bit suffix ids, 2048, 3072 or 4096
+                                   with 64-bit ones */
   int async;                    /* nonzero: calls return after enqueue when outputs are on the device */
   int timing;                   /* nonzero: record CUDA events around every phase (see cxbwt_stats) */
   int algorithm;                /* CXBWT_ALGO_*: how the suffixes are sorted (all give identical output) */
@@ -142,9 +144,9 @@ typedef struct {
  *             GROUPS when the reads are at most 528 bases, else LSD.
  *  LSD      - stable LSD radix passes over every 4-base digit of the
  *             A-padded suffixes (Section 3.2 as stated: one pass per digit).
- *  GROUPS   - LSD passes over the first l = 16 (or prefix_len = 12)
- *             bases only (the l-prefix partition of Section 3.1), then each
- *             group of suffixes sharing those bases is finished on chip. */
+ *  GROUPS   - LSD passes over the first l bases only (prefix_len: 16, 12 or,
+ *             in small builds, 8; the l-prefix partition of Section 3.1), then
+ *             each group of suffixes sharing those bases is finished on chip. */
 #define CXBWT_ALGO_AUTO 0
 #define CXBWT_ALGO_LSD 1
 #define CXBWT_ALGO_GROUPS 2
@@ -167,7 +169,7 @@ typedef struct {
   double group_ms;              /* device time finishing groups (group plan, only with `timing`) */
   double emit_ms;               /* device time of the emission (only with `timing`) */
   uint64_t slices;              /* device-memory-bounded slices sorted (one per build when it fits) */
-  uint64_t cta_groups;          /* groups of equal first 16 bases finished by one CTA (33 .. 2048 rows) */
+  uint64_t cta_groups;          /* groups of equal first l bases finished by one CTA (33 .. 2048 rows) */
   uint64_t big_groups;          /* larger groups, finished with more digit passes */
   uint64_t carried_pass_launches; /* digit passes (among sort_pass_launches) that load the key window the
                                      previous pass carried, instead of generating ids or gathering it */

@@ -314,7 +314,7 @@ int sort_slice(cxbwt_ctx* c, Run& r, const Slice& sl, int* cur_out, cudaEvent_t*
   }
   for (int64_t w = int64_t(pl.w_last); w >= 0; --w) {
     // The group plan sorts the first l = depth bases of window 0 (4 bases per
-    // digit): 4 passes for l = 16, 3 for l = 12.
+    // digit): 4 passes for l = 16, 3 for l = 12, 2 for l = 8.
     const uint32_t w_digits = (pl.groups && w == 0) ? pl.depth / 4 : 4u;
     const uint32_t d_lo = uint32_t(4 * w);
     const uint32_t d_hi = std::min<uint32_t>(d_lo + w_digits - 1, pl.D - 1);

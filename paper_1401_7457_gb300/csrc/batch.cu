@@ -82,7 +82,7 @@ int build_pack(cxbwt_ctx* c, const cxbwt_collection* colls, const std::vector<ui
   pl.len_passes = 0;
   pl.n_words = words;
   // The group plan's depth l: the option, else the autotuned one for the
-  // pack's size class, else 16 (16 also when l = 12 leaves too many bases).
+  // pack's size class, else by its size (16 also when another leaves too many bases).
   int depth = c->opt.prefix_len;
   {
     int t_tile = 0, t_algo = 0, t_depth = 0;

@@ -26,7 +26,7 @@ struct SegArgs {
   void* vals;             // suffix ids (uint32 or uint64), sorted by that window; finished in place
   uint32_t n_items;
   ReadIndex R;
-  uint32_t depth;         // bases already sorted: l of the group plan (12 or 16)
+  uint32_t depth;         // bases already sorted: l of the group plan (8, 12 or 16)
   uint32_t key_mask;      // the window bits of those bases: rows are in one group when their masked keys are equal
   uint2* cta_list;        // (first row, rows) of remainders of 33 .. kCtaMax rows
   uint32_t cta_cap;

@@ -179,7 +179,7 @@ struct Plan {
   int idb = 4;            // suffix id bytes
   uint32_t sym = 0;       // id bits holding the preceding base (0 or 2)
   bool groups = false;
-  uint32_t depth = 16;    // group plan: bases sorted by the LSD passes (l of Section 3.1: 12 or 16)
+  uint32_t depth = 16;    // group plan: bases sorted by the LSD passes (l of Section 3.1: 8, 12 or 16)
   int seg_words = 0;
   uint32_t w_last = 0;    // windows [0, w_last] are sorted by LSD passes over all rows of a slice
 };

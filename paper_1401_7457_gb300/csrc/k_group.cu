@@ -1,5 +1,5 @@
 // Finishing the sort inside groups of suffixes that share their first l
-// bases (l = 16, or 12: the depth of the group plan).
+// bases (l = 16, 12 or 8: the depth of the group plan).
 //
 // After the stable LSD passes over the first l bases of the 16-base window,
 // the suffix ids are ordered by those bases (A-padded) and, among equal
