@@ -82,3 +82,22 @@ def test_merge_plan_for_parts(n, length, share, merged):
     assert torch.equal(got[:(N + 15) // 16], want[0])
     none = torch.full_like(d, -1)
     assert torch.equal(torch.where(dollar == none, d, dollar), want[1]) and torch.equal(cnt + k, want[2])
+
+
+@pytest.mark.parametrize("n,length", [(20_164, 12), (20_166, 12), (65_536, 15), (65_537, 15), (80_000, 13), (70_000, 16),
+                                      (17_476, 14), (17_477, 14), (80_000, 17)])
+def test_group_plan_depth_by_size(n, length):
+    """Either side of the lines between l = 8, 12 and 16, for reads of 12 to 17
+    bases: the LSD plan's result, with and without a context."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1401_7457_gb300 import binding
+    words, lens = reads(n, length)
+    with binding.Context(device=0) as c, binding.Context(device=0, algorithm=binding.Context.ALGO_LSD) as lsd:
+        got, want = c.build(words, lens), lsd.build(words, lens)
+        assert c.stats()["merge_launches"] == 0
+    out = [torch.zeros_like(t) for t in want[:3]]
+    binding.build_noalloc(words, lens.cpu().numpy().view("uint32"), *out)
+    torch.cuda.synchronize()
+    for a, b, d in zip(got[:3], want[:3], out):
+        assert torch.equal(a, b) and torch.equal(d, b)
